@@ -291,7 +291,8 @@ int esdc_collocation(esdc_handle* h, double* y_out, double* r_out, void* stream)
  * (ionic model + quadrature), 2 = diffusion solve (CG), 3 = residual.
  * esdc_profile_read returns, per class, the summed milliseconds ms[4] and the
  * number of launches launches[4] since the last read, then resets them; it
- * synchronises the recorded events.  Not part of the method; no effect on results.
+ * synchronises the recorded events.  A step that runs as one launch (small meshes)
+ * counts under class 1.  Not part of the method; no effect on results.
  */
 int esdc_profile(esdc_handle* h, int enable);
 int esdc_profile_read(esdc_handle* h, double* ms, long long* launches);
@@ -398,9 +399,10 @@ int esdc_table_errors(int model, const double* params, int n_params, int M, doub
  * microseconds (0: the normal 1 s) have passed, raises the TIMEOUT flag and
  * returns.  The solve's result, and the state of a sweep that ran such solves,
  * are then undefined, and esdc_diffusion_solve / esdc_residual return
- * ESDC_ERR_DEVICE_TIMEOUT.  skip_block < 0 restores normal operation.  Only the
+ * ESDC_ERR_DEVICE_TIMEOUT.  skip_block < 0 restores normal operation.  The
  * Chebyshev and CG solves have grid barriers (options.solver 1 and 3, and 0
- * where it does not take the DCT).  Synchronises the device.  Returns
+ * where it does not take the DCT), and so have the steps that small meshes take as
+ * one launch, whatever their solver.  Synchronises the device.  Returns
  * ESDC_OK, ESDC_ERR_INVALID_ARG (null handle, limit_us above 1e6) or
  * ESDC_ERR_CUDA.
  */

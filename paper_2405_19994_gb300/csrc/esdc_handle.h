@@ -65,6 +65,12 @@ struct esdc_handle {
            *LAMN = nullptr, *rhs = nullptr, *R = nullptr, *ydev = nullptr, *Vprev = nullptr;
     CgWork cg{};
     DctDev dct{};                         // options.solver = 2
+    SmallDev small;                       // one-launch steps of small meshes
+    // rmax, flags, cg_log and the barrier words in one allocation, so that one
+    // memset of ctl_bytes clears what a step accumulates into (not the
+    // barrier's two test words, which follow)
+    void* ctl = nullptr;
+    size_t ctl_bytes = 0;
     // adjoint recording (set only inside esdc_adjoint_backward): Y^{1..K},
     // G^{0..K}, FI^{0..K} of one step, each block [M][NS][ld] or [M][ld]
     double *tapeY = nullptr, *tapeG = nullptr, *tapeFI = nullptr;
@@ -86,6 +92,16 @@ struct esdc_handle {
     long long prof_cnt[ESDC_PROF_CLASSES] = {};
     char err[256] = {0};
 };
+// One-launch steps of small meshes (esdc_small.cuh).  prepare: workspace and
+// matrices at creation when the mesh qualifies.  step: launches the step and sets
+// *taken, or leaves it to the launch sequence.
+cudaError_t esdc_small_prepare(esdc_handle* h);
+void esdc_small_destroy(SmallDev* d);
+cudaError_t esdc_small_step(esdc_handle* h, StepArgs& a, double* y, int M, int K, cudaStream_t s, bool* taken);
+cudaError_t esdc_small_launch_hh(const StepArgs& a, const void* args, int M, int blocks, int threads, size_t smem,
+                                 cudaStream_t s);
+cudaError_t esdc_small_launch_syn(const StepArgs& a, const void* args, int M, int blocks, int threads, size_t smem,
+                                  cudaStream_t s);
 // (Re)builds the handle's gate table for its current parameters (esdc_step.cu).
 cudaError_t esdc_vtab_upload(esdc_handle* h);
 

@@ -149,6 +149,22 @@ struct DctDev {
     size_t yzy_smem = 0;
 };
 
+// The one-launch step of small meshes (esdc_small.cuh): dense cosine matrices of
+// an axis in the parity-split form.
+struct SmallAxis {
+    int n, hp;                       // length, (n + 1) / 2
+    const double* F;                 // [hp][n]: cos(pi k (2 i + 1)/(2 n)), row i < hp, column k
+    const double* B;                 // [n][hp]: c_k cos(pi k (2 i + 1)/(2 n)), c_0 = 1, c_k = 2, row k, column i < hp
+};
+struct SmallDev {
+    void* part = nullptr;            // partial sums' cells [4][SMs]; nullptr: the mesh is not small
+    void* cells = nullptr;           // the nodes' exchange cells [2 or 7][N]
+    double* mats = nullptr;          // the axes' matrices; nullptr: no dense DCT for this mesh
+    double* winv = nullptr;          // [M_max][ld]
+    SmallAxis ax[3] = {};
+    int mat_doubles = 0;
+};
+
 // CG solve on the handle's mesh: (I - g L) x = b (Jacobi-preconditioned).
 struct CgWork {
     double *r, *p, *q, *z;          // [ld] each

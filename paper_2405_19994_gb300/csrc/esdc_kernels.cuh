@@ -295,22 +295,18 @@ __device__ __forceinline__ void setup_iter_body(const StepArgs& a, const PhaseAr
     }
 }
 
+// The set-up of a node in two parts that touch different rows: the V row with
+// the auxiliaries (lap_vn = L V_n at the node), and one gate.
 template <class Model, int M, bool MIXED>
-__device__ __forceinline__ void setup_body(const StepArgs& a, const PhaseArgs& ph, const MeshDev& m,
-                                           const StimDev& st, const unsigned* on, double D, int p, int ix, int iy,
-                                           int iz)
+__device__ __forceinline__ void setup_v(const StepArgs& a, const PhaseArgs& ph, const StimDev& st, const unsigned* on,
+                                        double D, double lap_vn, const double (&u)[Model::NS],
+                                        const float (&uf)[Model::NS], int p, int ix, int iy, int iz)
 {
-    constexpr int NS = Model::NS, NA = Model::NA, NG = Model::NG;
+    constexpr int NS = Model::NS, NA = Model::NA;
     const int64_t ld = a.m.ld;
-    double u[NS];
-#pragma unroll
-    for (int s = 0; s < NS; ++s) u[s] = a.yn[s * ld + p];
-    const double fi = D * lap(m, a.yn, p, ix, iy, iz);
+    const double fi = D * lap_vn;
     double mI, ha[NA > 0 ? NA : 1];
-    float uf[NS];
     if (MIXED) {
-#pragma unroll
-        for (int s = 0; s < NS; ++s) uf[s] = (float)u[s];
         float mIf, haf[NA > 0 ? NA : 1];
         Model::currents_f(a.mpf.p, uf, mIf, haf);
         mI = mIf;
@@ -329,29 +325,54 @@ __device__ __forceinline__ void setup_body(const StepArgs& a, const PhaseArgs& p
         for (int s = 1; s <= NA; ++s) { Gj[s * ld + p] = ha[s - 1]; Yj[s * ld + p] = u[s]; }
         a.FI[(int64_t)j * ld + p] = fi;
     }
+}
+
+template <class Model, int M, bool MIXED>
+__device__ __forceinline__ void setup_gate(const StepArgs& a, const PhaseArgs& ph, int g, double V, float Vf,
+                                           const typename Model::VCtx& vc, int p)
+{
+    constexpr int NS = Model::NS, NA = Model::NA, NG = Model::NG;
+    const int64_t ld = a.m.ld;
+    const int s = 1 + NA + g;
+    const double us = a.yn[s * ld + p];
+    double lam, g0;                          // g0 = Lambda (u - w_inf) = Lambda u + b
+    if (MIXED) {
+        float lf, yf;
+        Model::gate_f(a.mpf.p, g, Vf, lf, yf);
+        lam = lf;
+        g0 = lam * (us - (double)yf);
+    } else {
+        double b;
+        Model::gate_lb(a.mp.p, vc, g, V, lam, b);
+        g0 = fma(lam, us, b);
+    }
+#pragma unroll
+    for (int j = 0; j < M; ++j) {
+        ph.Gnew[((int64_t)j * NS + s) * ld + p] = g0;
+        a.Y[((int64_t)j * NS + s) * ld + p] = us;
+    }
+    gate_tables<M>(a, g, NG, lam, p);
+}
+
+template <class Model, int M, bool MIXED>
+__device__ __forceinline__ void setup_body(const StepArgs& a, const PhaseArgs& ph, const MeshDev& m,
+                                           const StimDev& st, const unsigned* on, double D, int p, int ix, int iy,
+                                           int iz)
+{
+    constexpr int NS = Model::NS, NG = Model::NG;
+    const int64_t ld = a.m.ld;
+    double u[NS];
+    float uf[NS] = {};
+#pragma unroll
+    for (int s = 0; s < NS; ++s) u[s] = a.yn[s * ld + p];
+    if (MIXED) {
+#pragma unroll
+        for (int s = 0; s < NS; ++s) uf[s] = (float)u[s];
+    }
+    setup_v<Model, M, MIXED>(a, ph, st, on, D, lap(m, a.yn, p, ix, iy, iz), u, uf, p, ix, iy, iz);
     const typename Model::VCtx vc = Model::vctx(a.mp, u[0]);
 #pragma unroll 1
-    for (int g = 0; g < NG; ++g) {
-        const int s = 1 + NA + g;
-        const double us = a.yn[s * ld + p];
-        double lam, g0;                          // g0 = Lambda (u - w_inf) = Lambda u + b
-        if (MIXED) {
-            float lf, yf;
-            Model::gate_f(a.mpf.p, g, uf[0], lf, yf);
-            lam = lf;
-            g0 = lam * (us - (double)yf);
-        } else {
-            double b;
-            Model::gate_lb(a.mp.p, vc, g, u[0], lam, b);
-            g0 = fma(lam, us, b);
-        }
-#pragma unroll
-        for (int j = 0; j < M; ++j) {
-            ph.Gnew[((int64_t)j * NS + s) * ld + p] = g0;
-            a.Y[((int64_t)j * NS + s) * ld + p] = us;
-        }
-        gate_tables<M>(a, g, NG, lam, p);
-    }
+    for (int g = 0; g < NG; ++g) setup_gate<Model, M, MIXED>(a, ph, g, u[0], uf[0], vc, p);
 }
 
 #ifndef ESDC_SETUP_MINBLOCKS
@@ -369,41 +390,48 @@ __device__ __forceinline__ void setup_body(const StepArgs& a, const PhaseArgs& p
 #endif
 // TAU: batched kernels may add the FAS correction tau (a.tau, rows 1..M; the
 // recursive form adds tau_i - tau_{i-1}, tau_0 = 0, to every row of node i).
-template <class Model, int M, bool MIXED, bool TAU = false>
-__device__ __forceinline__ void node_body(const StepArgs& a, const PhaseArgs& ph, const MeshDev& m,
-                                          const StimDev& st, const unsigned* on, double D, int p, int ix, int iy,
-                                          int iz)
+// R0: hands the V row's right-hand side b, its initial guess x and the residual
+// r = b - (I - dt d_i D L) x to the caller instead of storing b.  D L x is the
+// same combination of stored f_I values as x is of potentials (f_I is linear in
+// V), so the residual needs no stencil on the guess.
+struct NodeSolve {
+    double b, x, r;
+};
+// A node evaluation in two parts that touch different rows (the gates enter the
+// V row only as values u of y_{i-1}): the V row with the auxiliaries, and one gate.
+// dtau: the FAS correction's difference tau_i - tau_{i-1} of state s.
+template <class Model, int M, bool TAU>
+__device__ __forceinline__ double node_dtau(const StepArgs& a, int ii, int s, int p)
 {
-    constexpr int NS = Model::NS, NA = Model::NA, NG = Model::NG;
+    constexpr int NS = Model::NS;
+    const int64_t ld = a.m.ld;
+    if (!TAU || !a.tau) return 0.0;
+    const double t1 = a.tau[((int64_t)ii * NS + s) * ld + p];
+    return ii > 0 ? t1 - a.tau[((int64_t)(ii - 1) * NS + s) * ld + p] : t1;
+}
+
+// lap_v: L V_{i-1} at the node, called only for i >= 2.
+template <class Model, int M, bool MIXED, bool TAU, bool R0, class Lap>
+__device__ __forceinline__ void node_v(const StepArgs& a, const PhaseArgs& ph, const StimDev& st, const unsigned* on,
+                                       double D, Lap lap_v, const double (&u)[Model::NS], const float (&uf)[Model::NS],
+                                       int p, int ix, int iy, int iz, NodeSolve* so)
+{
+    constexpr int NS = Model::NS, NA = Model::NA;
     const int64_t ld = a.m.ld;
     const int i = ph.i;
     const bool eval = i >= 2;                 // G at y_{i-1}^{k+1}
     const bool quad = i <= M;                 // explicit rows of y_i^{k+1}
     const int jm = i - 2;                     // 0-based index of node i-1
     const int ii = i - 1;                     // 0-based index of node i
-    auto dtau = [&](int s) -> double {
-        if (!TAU || !a.tau) return 0.0;
-        const double t1 = a.tau[((int64_t)ii * NS + s) * ld + p];
-        return ii > 0 ? t1 - a.tau[((int64_t)(ii - 1) * NS + s) * ld + p] : t1;
-    };
-    const double* src = eval ? a.Y + (int64_t)jm * NS * ld : a.yn;   // y_{i-1}^{k+1}
-    double u[NS];
-#pragma unroll
-    for (int s = 0; s < NS; ++s) u[s] = src[s * ld + p];
     const double* Gp = ph.Gold + (int64_t)jm * NS * ld;               // G_{i-1}^k
     double* Gq = ph.Gnew + (int64_t)jm * NS * ld;                     // G_{i-1}^{k+1}
     double* Yi = a.Y + (int64_t)ii * NS * ld;
     const double dtd = quad ? a.dtd[i] : 0.0;
-
-    // ---- V row and auxiliaries
-    double dlt0 = 0.0, ha[NA > 0 ? NA : 1];
-    float uf[NS];
+    double dlt0 = 0.0, dfi = 0.0, ha[NA > 0 ? NA : 1];
     if (eval) {
-        const double fi = D * lap(m, src, p, ix, iy, iz);
+        const double fi = D * lap_v();
         double mI;
         if (MIXED) {                      // precision form: the ionic model in FP32
-#pragma unroll
-            for (int s = 0; s < NS; ++s) uf[s] = (float)u[s];
             float mIf, haf[NA > 0 ? NA : 1];
             Model::currents_f(a.mpf.p, uf, mIf, haf);
             mI = mIf;
@@ -417,6 +445,7 @@ __device__ __forceinline__ void node_body(const StepArgs& a, const PhaseArgs& ph
         a.FI[(int64_t)jm * ld + p] = fi;
         Gq[p] = fi + fE;
         dlt0 = fE - (Gp[p] - fi_old);
+        if (R0) dfi = fi - fi_old;
 #pragma unroll
         for (int s = 1; s <= NA; ++s) Gq[s * ld + p] = ha[s - 1];
     }
@@ -424,15 +453,25 @@ __device__ __forceinline__ void node_body(const StepArgs& a, const PhaseArgs& ph
         // Initial guess of the V_i solve: V_i^k moved by the change the previous
         // node just received, V_i^k + rho (V_{i-1}^{k+1} - V_{i-1}^k).  Only the
         // starting point of CG changes; the solution is the same.
-        const double vik = Yi[p];
-        if (eval) Yi[p] = fma(ph.rho, u[0] - a.Vprev[p], vik);
+        const double vik = Yi[p], fik = a.FI[(int64_t)ii * ld + p];
+        double xw = vik;
+        if (eval) {
+            xw = fma(ph.rho, u[0] - a.Vprev[p], vik);
+            Yi[p] = xw;
+        }
         a.Vprev[p] = vik;
         double q = u[0];
 #pragma unroll
         for (int j = 0; j < M; ++j) q = fma(a.dS0[ii][j], ph.Gold[(int64_t)j * NS * ld + p], q);
-        double rv = fma(dtd, dlt0 - a.FI[(int64_t)ii * ld + p], q);
-        if (TAU) rv += dtau(0);                // (x + 0.0 is not x in IEEE arithmetic: no add without TAU)
-        a.rhs[p] = rv;
+        double rv = fma(dtd, dlt0 - fik, q);
+        if (TAU) rv += node_dtau<Model, M, TAU>(a, ii, 0, p);   // (x + 0.0 is not x in IEEE arithmetic: no add without TAU)
+        if (R0) {
+            so->b = rv;
+            so->x = xw;
+            so->r = fma(dtd, fma(ph.rho, dfi, fik), rv - xw);
+        } else {
+            a.rhs[p] = rv;
+        }
 #pragma unroll
         for (int s = 1; s <= NA; ++s) {
             const double dl = eval ? ha[s - 1] - Gp[s * ld + p] : 0.0;
@@ -440,44 +479,75 @@ __device__ __forceinline__ void node_body(const StepArgs& a, const PhaseArgs& ph
 #pragma unroll
             for (int j = 0; j < M; ++j) qa = fma(a.dS0[ii][j], ph.Gold[((int64_t)j * NS + s) * ld + p], qa);
             double ya = fma(dtd, dl, qa);
-            if (TAU) ya += dtau(s);
+            if (TAU) ya += node_dtau<Model, M, TAU>(a, ii, s, p);
             Yi[s * ld + p] = ya;
         }
     }
-    // ---- gates, one at a time
+}
+
+template <class Model, int M, bool MIXED, bool TAU>
+__device__ __forceinline__ void node_gate(const StepArgs& a, const PhaseArgs& ph, int g, double us, double V, float Vf,
+                                          const typename Model::VCtx& vc, int p)
+{
+    constexpr int NS = Model::NS, NA = Model::NA, NG = Model::NG;
+    const int64_t ld = a.m.ld;
+    const int i = ph.i, jm = i - 2, ii = i - 1, s = 1 + NA + g;
+    const bool eval = i >= 2, quad = i <= M;
+    const double* Gp = ph.Gold + (int64_t)jm * NS * ld;
+    double* Gq = ph.Gnew + (int64_t)jm * NS * ld;
+    double* Yi = a.Y + (int64_t)ii * NS * ld;
+    double dl = 0.0;
+    if (eval) {
+        // g_n = Lambda(V) u + b(V) + Lambda_n (u_n - u), b = -Lambda w_inf
+        const double ln = a.LAMN[(int64_t)g * ld + p], du = a.yn[s * ld + p] - us;
+        double gn;
+        if (MIXED) {
+            float lf, yf;
+            Model::gate_f(a.mpf.p, g, Vf, lf, yf);
+            gn = (double)lf * (us - (double)yf) + ln * du;
+        } else {
+            double lam, b;
+            Model::gate_lb(a.mp.p, vc, g, V, lam, b);
+            gn = fma(ln, du, fma(lam, us, b));
+        }
+        Gq[s * ld + p] = gn;
+        dl = gn - Gp[s * ld + p];
+    }
+    if (quad) {
+        double qg = us;
+#pragma unroll
+        for (int j = 0; j < M; ++j)
+            qg = fma(a.S[(((int64_t)ii * M + j) * NG + g) * ld + p],
+                     ph.Gold[((int64_t)j * NS + s) * ld + p], qg);
+        double yg = fma(a.PHI[((int64_t)ii * NG + g) * ld + p], dl, qg);
+        if (TAU) yg += node_dtau<Model, M, TAU>(a, ii, s, p);
+        Yi[s * ld + p] = yg;
+    }
+}
+
+template <class Model, int M, bool MIXED, bool TAU = false>
+__device__ __forceinline__ void node_body(const StepArgs& a, const PhaseArgs& ph, const MeshDev& m,
+                                          const StimDev& st, const unsigned* on, double D, int p, int ix, int iy,
+                                          int iz)
+{
+    constexpr int NS = Model::NS, NA = Model::NA, NG = Model::NG;
+    const int64_t ld = a.m.ld;
+    const bool eval = ph.i >= 2;
+    const double* src = eval ? a.Y + (int64_t)(ph.i - 2) * NS * ld : a.yn;   // y_{i-1}^{k+1}
+    double u[NS];
+    float uf[NS];
+#pragma unroll
+    for (int s = 0; s < NS; ++s) u[s] = src[s * ld + p];
+    if (MIXED && eval) {
+#pragma unroll
+        for (int s = 0; s < NS; ++s) uf[s] = (float)u[s];
+    }
+    node_v<Model, M, MIXED, TAU, false>(a, ph, st, on, D, [&]() { return lap(m, src, p, ix, iy, iz); }, u, uf, p, ix,
+                                        iy, iz, nullptr);
     typename Model::VCtx vc{};
     if (eval && !MIXED) vc = Model::vctx(a.mp, u[0]);
 #pragma unroll
-    for (int g = 0; g < NG; ++g) {
-        const int s = 1 + NA + g;
-        double dl = 0.0;
-        if (eval) {
-            // g_n = Lambda(V) u + b(V) + Lambda_n (u_n - u), b = -Lambda w_inf
-            const double ln = a.LAMN[(int64_t)g * ld + p], du = a.yn[s * ld + p] - u[s];
-            double gn;
-            if (MIXED) {
-                float lf, yf;
-                Model::gate_f(a.mpf.p, g, uf[0], lf, yf);
-                gn = (double)lf * (u[s] - (double)yf) + ln * du;
-            } else {
-                double lam, b;
-                Model::gate_lb(a.mp.p, vc, g, u[0], lam, b);
-                gn = fma(ln, du, fma(lam, u[s], b));
-            }
-            Gq[s * ld + p] = gn;
-            dl = gn - Gp[s * ld + p];
-        }
-        if (quad) {
-            double qg = u[s];
-#pragma unroll
-            for (int j = 0; j < M; ++j)
-                qg = fma(a.S[(((int64_t)ii * M + j) * NG + g) * ld + p],
-                         ph.Gold[((int64_t)j * NS + s) * ld + p], qg);
-            double yg = fma(a.PHI[((int64_t)ii * NG + g) * ld + p], dl, qg);
-            if (TAU) yg += dtau(s);
-            Yi[s * ld + p] = yg;
-        }
-    }
+    for (int g = 0; g < NG; ++g) node_gate<Model, M, MIXED, TAU>(a, ph, g, u[1 + NA + g], u[0], uf[0], vc, p);
 }
 
 // Node 1 of the next sweep fused into a launch (a.fuse1, M >= 2): the explicit
@@ -642,6 +712,26 @@ inline int resident_grid(const esdc_handle* h, int per_sm, int threads)
     return (int)(need < cap ? (need < 1 ? 1 : need) : cap);
 }
 
+// The constants of a step on M nodes: dt S_ij(0), dt B_ijk, dt d_i and the
+// stimulus boxes that are on at each collocation time.
+inline void step_constants(const esdc_handle* h, StepArgs& a, int M)
+{
+    const ColloData* C = &h->col[M - 1];
+    for (int i = 0; i < M; ++i)
+        for (int j = 0; j < M; ++j) {
+            a.dS0[i][j] = a.dt * C->S0[i][j];
+            for (int q = 0; q < M; ++q) a.dtB[i][j][q] = a.dt * C->B[i][j][q];
+        }
+    for (int i = 0; i <= M; ++i) {
+        a.dtd[i] = a.dt * C->d[i];
+        const double tj = a.t_n + C->c[i] * a.dt;
+        unsigned on = 0;
+        for (int b = 0; b < h->stim.nbox; ++b)
+            if (tj >= h->stim.t_on[b] && tj < h->stim.t_off[b]) on |= 1u << b;
+        a.stim_on[i] = on;
+    }
+}
+
 template <class Model, int M, bool MIXED>
 cudaError_t launch_step_kernels(esdc_handle* h, StepArgs& a, double* y, int K, cudaStream_t s)
 {
@@ -658,19 +748,7 @@ cudaError_t launch_step_kernels(esdc_handle* h, StepArgs& a, double* y, int K, c
     const double g0 = h->D;   // operator scale: (I - dt d_i D L)
     const ColloData* C = &h->col[M - 1];
 
-    for (int i = 0; i < M; ++i)
-        for (int j = 0; j < M; ++j) {
-            a.dS0[i][j] = a.dt * C->S0[i][j];
-            for (int q = 0; q < M; ++q) a.dtB[i][j][q] = a.dt * C->B[i][j][q];
-        }
-    for (int i = 0; i <= M; ++i) {
-        a.dtd[i] = a.dt * C->d[i];
-        const double tj = a.t_n + C->c[i] * a.dt;
-        unsigned on = 0;
-        for (int b = 0; b < h->stim.nbox; ++b)
-            if (tj >= h->stim.t_on[b] && tj < h->stim.t_off[b]) on |= 1u << b;
-        a.stim_on[i] = on;
-    }
+    step_constants(h, a, M);
     a.Gnew = h->G0;
     a.Gold = h->G0;
     // Node 1 of each sweep runs inside the launch before it (the set-up, or the

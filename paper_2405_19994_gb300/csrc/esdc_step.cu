@@ -183,6 +183,7 @@ void free_all(esdc_handle* h)
     for (auto& e : h->prof_ev)
         if (e) cudaEventDestroy(e);
     esdc_dct_destroy(&h->dct);
+    esdc_small_destroy(&h->small);
     if (h->lay) cudaFree(h->lay);
     if (h->layf) cudaFree(h->layf);
     if (h->wdiag) cudaFree(h->wdiag);
@@ -191,8 +192,7 @@ void free_all(esdc_handle* h)
     esdc_ztab_free(h->zt);
     void* ptrs[] = {h->Y, h->G0, h->G1, h->FI, h->S, h->PHI, h->LAMN, h->rhs, h->R, h->ydev, h->Vprev,
                     h->cg.r, h->cg.p, h->cg.q, h->cg.z, h->cg.r32, h->cg.p32, h->cg.q32, h->cg.z32,
-                    h->cg.e32, h->cg.part, h->cg.bar, h->cg.status,
-                    h->rmax, h->flags, h->cg_log};
+                    h->cg.e32, h->cg.part, h->cg.status, h->ctl};
     for (void* p : ptrs)
         if (p) cudaFree(p);
 }
@@ -381,14 +381,21 @@ int esdc_create(const esdc_mesh* mesh, double sigma, double chi, double Cm, int 
     h->cg.threads = ESDC_CG_THREADS;
     h->cg.max_blocks = esdc_cg_blocks(h->mesh, h->cg.threads);
     if (h->cg.max_blocks < 1) return fail(ESDC_ERR_CUDA);
-    if (cudaMalloc((void**)&h->cg.part, sizeof(double) * 8 * h->cg.max_blocks) != cudaSuccess ||
-        cudaMalloc((void**)&h->cg.bar, sizeof(unsigned) * 4) != cudaSuccess ||
-        cudaMalloc((void**)&h->cg.status, sizeof(int) * 2) != cudaSuccess ||
-        cudaMalloc((void**)&h->rmax, sizeof(unsigned long long) * 2 * ESDC_NSMAX) != cudaSuccess ||
-        cudaMalloc((void**)&h->flags, sizeof(int)) != cudaSuccess ||
-        cudaMalloc((void**)&h->cg_log, sizeof(int) * 64 * ESDC_MMAX) != cudaSuccess)
-        return fail(ESDC_ERR_NO_MEMORY);
     h->cg_log_len = 64 * ESDC_MMAX;
+    // rmax [2 NSMAX] | flags, pad | log | barrier count, spare | its two test words
+    const size_t rmax_b = sizeof(unsigned long long) * 2 * ESDC_NSMAX, flag_b = 8, log_b = sizeof(int) * h->cg_log_len;
+    h->ctl_bytes = rmax_b + flag_b + log_b + 2 * sizeof(unsigned);
+    if (cudaMalloc((void**)&h->cg.part, sizeof(double) * 8 * h->cg.max_blocks) != cudaSuccess ||
+        cudaMalloc((void**)&h->cg.status, sizeof(int) * 2) != cudaSuccess ||
+        cudaMalloc(&h->ctl, h->ctl_bytes + 2 * sizeof(unsigned)) != cudaSuccess)
+        return fail(ESDC_ERR_NO_MEMORY);
+    {
+        char* c = static_cast<char*>(h->ctl);
+        h->rmax = reinterpret_cast<unsigned long long*>(c);
+        h->flags = reinterpret_cast<int*>(c + rmax_b);
+        h->cg_log = reinterpret_cast<int*>(c + rmax_b + flag_b);
+        h->cg.bar = reinterpret_cast<unsigned*>(c + rmax_b + flag_b + log_b);
+    }
     if (o.precision == 1) {                       // FP32 vectors of the inner solves
         float** fv[] = {&h->cg.r32, &h->cg.p32, &h->cg.q32, &h->cg.z32, &h->cg.e32};
         for (float** f : fv) {
@@ -396,10 +403,8 @@ int esdc_create(const esdc_mesh* mesh, double sigma, double chi, double Cm, int 
             cudaMemset(*f, 0, sizeof(float) * ld);
         }
     }
-    cudaMemset(h->cg.bar, 0, sizeof(unsigned) * 4);
+    cudaMemset(h->ctl, 0, h->ctl_bytes + 2 * sizeof(unsigned));
     cudaMemset(h->cg.status, 0, sizeof(int) * 2);
-    cudaMemset(h->flags, 0, sizeof(int));
-    cudaMemset(h->cg_log, 0, sizeof(int) * h->cg_log_len);
     // the DCT-II tables: for the DCT solve itself (2) and for the automatic
     // choice on the FP64 path (0), which takes it while sigma is scalar and the
     // transforms are cheap (x and y; the fourth order, set later, adds z)
@@ -410,6 +415,10 @@ int esdc_create(const esdc_mesh* mesh, double sigma, double chi, double Cm, int 
         const cudaError_t e = esdc_dct_create(h->mesh, o.M_max, &h->dct);
         if (e != cudaSuccess) return fail(e == cudaErrorMemoryAllocation ? ESDC_ERR_NO_MEMORY : ESDC_ERR_CUDA);
         h->cg.dct = &h->dct;
+    }
+    {
+        const cudaError_t e = esdc_small_prepare(h);
+        if (e != cudaSuccess) return fail(e == cudaErrorMemoryAllocation ? ESDC_ERR_NO_MEMORY : ESDC_ERR_CUDA);
     }
     if (cudaDeviceSynchronize() != cudaSuccess) return fail(ESDC_ERR_CUDA);
     *out = h;
@@ -632,16 +641,17 @@ int esdc_sweep(esdc_handle* h, double* y, double t, double dt, int M, int K, voi
     if (K < 0 || K > 64) return set_err(h, ESDC_ERR_INVALID_ARG, "K=%d outside 0..64", K);
     if (!(dt > 0.0) || !std::isfinite(dt) || !std::isfinite(t)) return set_err(h, ESDC_ERR_INVALID_ARG, "bad t/dt");
     cudaStream_t s = (cudaStream_t)stream;
-    CUDA_TRY(h, cudaMemsetAsync(h->rmax, 0, sizeof(unsigned long long) * 2 * ESDC_NSMAX, s));
-    CUDA_TRY(h, cudaMemsetAsync(h->flags, 0, sizeof(int), s));
-    CUDA_TRY(h, cudaMemsetAsync(h->cg_log, 0, sizeof(int) * h->cg_log_len, s));
+    CUDA_TRY(h, cudaMemsetAsync(h->ctl, 0, h->ctl_bytes, s));   // rmax, flags, the log, the barrier count
     StepArgs a{};                        // value-initialised: every pointer null, every count 0
     a.m = h->mesh; a.st = h->stim; a.mp = h->mp; a.mpf = h->mpf;
     a.dt = dt; a.t_n = t; a.D = h->D; a.inv_Cm = 1.0 / h->Cm;
     a.yn = y; a.Y = h->Y; a.FI = h->FI; a.S = h->S; a.PHI = h->PHI; a.LAMN = h->LAMN; a.rhs = h->rhs;
     a.R = h->R; a.rmax = h->rmax; a.flags = h->flags; a.Vprev = h->Vprev;
-    cudaError_t e;
-    if (h->opt.precision == 1)
+    bool small = false;
+    cudaError_t e = esdc_small_step(h, a, y, M, K, s, &small);
+    if (e != cudaSuccess || small) {
+        // (an error falls through to the report below)
+    } else if (h->opt.precision == 1)
         e = esdc_dispatch_mixed(h, a, y, M, K, s);
     else
         e = h->model == ESDC_MODEL_HH1952 ? dispatch_M<esdc::HH1952, false>(h, a, y, M, K, s)
