@@ -1298,11 +1298,11 @@ int esdc_batch_create(int n, const esdc_mesh* meshes, const double* sigma, doubl
     b->chi = chi; b->Cm = Cm;
     b->mp = mp; b->mpf = mpf;
     {
-        std::vector<double> rows;
+        TableRows rows;
         double err[2];
         if (esdc_vtab_build(model, mp.p, rows, &err[0], &err[1]) == 0) {
-            if (cudaMalloc((void**)&b->vtab, sizeof(double) * rows.size()) != cudaSuccess ||
-                cudaMemcpy(b->vtab, rows.data(), sizeof(double) * rows.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+            if (cudaMalloc((void**)&b->vtab, sizeof(double) * rows->size()) != cudaSuccess ||
+                cudaMemcpy(b->vtab, rows->data(), sizeof(double) * rows->size(), cudaMemcpyHostToDevice) != cudaSuccess)
                 return fail(ESDC_ERR_NO_MEMORY);
             b->mp.vtab = b->vtab;
         }

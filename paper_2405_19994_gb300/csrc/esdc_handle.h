@@ -54,6 +54,7 @@ struct esdc_handle {
     ModelDevF mpf{};
     double sigma = 0, chi = 0, Cm = 0, D = 0;
     double* vtab = nullptr;                    // the gate table of the model (SYN19), see ModelDev
+    TableRows vtab_rows;                       // the table that vtab holds
     ZtabSlots zt;                              // set-up coefficient tables per (M, dt)
     double vtab_err[2] = {0, 0};               // its build-time errors (b / |Lambda| absolute, Lambda relative)
     double *lay = nullptr, *wdiag = nullptr;   // layered conductivity (see MeshDev)

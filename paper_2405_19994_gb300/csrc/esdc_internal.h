@@ -1,6 +1,7 @@
 // Internal declarations of the HSDC library (not part of the C ABI).
 #pragma once
 #include <cstdint>
+#include <memory>
 #include <vector>
 #include <cuda_runtime.h>
 
@@ -196,11 +197,13 @@ void esdc_dct_destroy(DctDev* d);
 cudaError_t esdc_dct_launch(const MeshDev& m, const CgWork& w, double g, const double* b, double* x,
                             int* iter_log, int* flags, cudaStream_t s);
 
+// A table's rows, shared with the process's cache of built tables.
+using TableRows = std::shared_ptr<const std::vector<double>>;
 // The gate table of a model (SYN19, HH1952): rows [ESDC_VTAB_N][ESDC_VTAB_ROW] and
 // the largest errors of its FP64 evaluation against the direct functions
 // (absolute for w_inf, relative for Lambda).  0: built; -1: no table for this
-// model; -2: an error above ESDC_VTAB_TOL (rows cleared).
-int esdc_vtab_build(int model, const double* params, std::vector<double>& rows, double* err_winf, double* err_lam);
+// model; -2: an error above ESDC_VTAB_TOL (no rows).
+int esdc_vtab_build(int model, const double* params, TableRows& rows, double* err_winf, double* err_lam);
 
 // The set-up's exponential coefficients tabulated in y = 1 - z, z = dt Lambda
 // (esdc_ztab.cpp): ESDC_ZTAB_OCT octaves of y, 2^ESDC_ZTAB_SUB intervals each,
@@ -217,9 +220,9 @@ int esdc_vtab_build(int model, const double* params, std::vector<double>& rows, 
 #define ESDC_ZTAB_ROW(M) (2 + (M) * ((M) + 1) * ESDC_ZTAB_NC)
 #define ESDC_ZTAB_TOL 4e-15         // refuse a table whose FP64 evaluation misses by more (units of dt)
 // Builds (or takes from this process's cache) the table for (M, dt, C);
-// returns 0, -1 (bad arguments) or -2 (error above ESDC_ZTAB_TOL, rows
-// cleared); *err: the largest error, in units of dt.
-int esdc_ztab_build(int M, double dt, const ColloData& C, std::vector<double>& rows, double* err);
+// returns 0, -1 (bad arguments) or -2 (error above ESDC_ZTAB_TOL, no
+// rows); *err: the largest error, in units of dt.
+int esdc_ztab_build(int M, double dt, const ColloData& C, TableRows& rows, double* err);
 // Device copies of the set-up tables of a handle or batch for a few (M, dt).
 #define ESDC_ZTAB_SLOTS 4
 struct ZtabSlots {

@@ -206,25 +206,25 @@ const double* esdc_ztab_device(ZtabSlots& z, int M, double dt, const ColloData& 
     if (z.builds >= ESDC_ZTAB_BUILDS) return nullptr;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return nullptr;
-    std::vector<double> rows;
+    TableRows rows;
     double err = 0.0;
     if (esdc_ztab_build(M, dt, C, rows, &err) != 0) return nullptr;
     const int k = z.next;
     z.next = (z.next + 1) % ESDC_ZTAB_SLOTS;
     // the slot may hold a table that kernels in flight read
     if (cudaDeviceSynchronize() != cudaSuccess) return nullptr;
-    if (z.n[k] < rows.size()) {
+    if (z.n[k] < rows->size()) {
         if (z.dev[k]) cudaFree(z.dev[k]);
         z.dev[k] = nullptr;
         z.n[k] = 0;
-        if (cudaMalloc((void**)&z.dev[k], sizeof(double) * rows.size()) != cudaSuccess) {
+        if (cudaMalloc((void**)&z.dev[k], sizeof(double) * rows->size()) != cudaSuccess) {
             z.dev[k] = nullptr;
             return nullptr;
         }
-        z.n[k] = rows.size();
+        z.n[k] = rows->size();
     }
     z.M[k] = 0;
-    if (cudaMemcpy(z.dev[k], rows.data(), sizeof(double) * rows.size(), cudaMemcpyHostToDevice) != cudaSuccess)
+    if (cudaMemcpy(z.dev[k], rows->data(), sizeof(double) * rows->size(), cudaMemcpyHostToDevice) != cudaSuccess)
         return nullptr;
     z.M[k] = M;
     z.dt[k] = dt;
@@ -243,17 +243,25 @@ void esdc_ztab_free(ZtabSlots& z)
 // The gate table of the handle's model for the parameters in h->mp (built on
 // the host, copied into h->vtab, allocated on first use); h->mp.vtab points
 // to it, or stays nullptr (direct evaluation) for models without a table or a
-// table that missed its accuracy check.  Synchronises the device before it
-// overwrites a table that kernels in flight may read.
+// table that missed its accuracy check.  The device's table stays while the
+// handle's table is the same one (a fit that varies the maximal conductances
+// sets parameters before every run; the 24 MB copy and its two host copies took
+// 3 ms a call).  Synchronises the device before it overwrites a table that
+// kernels in flight may read.
 cudaError_t esdc_vtab_upload(esdc_handle* h)
 {
-    std::vector<double> rows;
+    TableRows rows;
     h->mp.vtab = nullptr;
     if (esdc_vtab_build(h->model, h->mp.p, rows, &h->vtab_err[0], &h->vtab_err[1]) != 0) return cudaSuccess;
     cudaError_t e = cudaSuccess;
-    if (!h->vtab) e = cudaMalloc((void**)&h->vtab, sizeof(double) * rows.size());
-    else e = cudaDeviceSynchronize();
-    if (e == cudaSuccess) e = cudaMemcpy(h->vtab, rows.data(), sizeof(double) * rows.size(), cudaMemcpyHostToDevice);
+    if (rows != h->vtab_rows) {
+        h->vtab_rows.reset();
+        if (!h->vtab) e = cudaMalloc((void**)&h->vtab, sizeof(double) * rows->size());
+        else e = cudaDeviceSynchronize();
+        if (e == cudaSuccess)
+            e = cudaMemcpy(h->vtab, rows->data(), sizeof(double) * rows->size(), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) h->vtab_rows = rows;
+    }
     if (e == cudaSuccess) h->mp.vtab = h->vtab;
     return e;
 }
@@ -806,7 +814,7 @@ int esdc_table_errors(int model, const double* params, int n_params, int M, doub
     if (need < 0 || n_params != need) return ESDC_ERR_INVALID_ARG;
     for (int k = 0; k < n_params; ++k)
         if (!std::isfinite(params[k])) return ESDC_ERR_INVALID_ARG;
-    std::vector<double> rows;
+    TableRows rows;
     if (esdc_vtab_build(model, params, rows, &err[0], &err[1]) == -1) return ESDC_ERR_INVALID_ARG;
     ColloData C;
     if (esdc_colloc_build(M, &C) != 0) return ESDC_ERR_INVALID_ARG;

@@ -158,7 +158,8 @@ void build_rows(int model, const double* params, int i0, int i1, double* out, do
 // that handles of the same model and a change of conductances reuse them.
 struct Cached {
     int model;
-    std::vector<double> key, rows;
+    std::vector<double> key;
+    TableRows rows;
     double ew, el;
 };
 std::mutex g_cache_mu;
@@ -167,9 +168,9 @@ constexpr size_t kCacheSize = 8;
 
 }  // namespace
 
-int esdc_vtab_build(int model, const double* params, std::vector<double>& rows, double* err_winf, double* err_lam)
+int esdc_vtab_build(int model, const double* params, TableRows& rows, double* err_winf, double* err_lam)
 {
-    rows.clear();
+    rows.reset();
     if (model != ESDC_MODEL_SYN19 && model != ESDC_MODEL_HH1952) return -1;
     const std::vector<double> key = model == ESDC_MODEL_SYN19 ? std::vector<double>(params, params + 72)
                                                                : std::vector<double>{params[6]};
@@ -190,7 +191,7 @@ int esdc_vtab_build(int model, const double* params, std::vector<double>& rows, 
             }
     }
     if (!hit) {
-        rows.assign((size_t)ESDC_VTAB_N * ESDC_VTAB_ROW, 0.0);
+        std::vector<double> v((size_t)ESDC_VTAB_N * ESDC_VTAB_ROW, 0.0);
         // rows are independent: split them over the host's cores; the maxima
         // do not depend on the split
         unsigned nt = std::thread::hardware_concurrency();
@@ -201,9 +202,10 @@ int esdc_vtab_build(int model, const double* params, std::vector<double>& rows, 
         for (unsigned t = 0; t < nt; ++t) {
             const int i0 = (int)t * per, i1 = std::min(ESDC_VTAB_N, i0 + per);
             if (i0 >= i1) break;
-            th.emplace_back(build_rows, model, params, i0, i1, rows.data(), std::ref(tw[t]), std::ref(tl[t]));
+            th.emplace_back(build_rows, model, params, i0, i1, v.data(), std::ref(tw[t]), std::ref(tl[t]));
         }
         for (auto& x : th) x.join();
+        rows = std::make_shared<const std::vector<double>>(std::move(v));
         for (unsigned t = 0; t < nt; ++t) {
             ew = std::fmax(ew, tw[t]);
             el = std::fmax(el, tl[t]);
@@ -215,7 +217,7 @@ int esdc_vtab_build(int model, const double* params, std::vector<double>& rows, 
     if (err_winf) *err_winf = ew;
     if (err_lam) *err_lam = el;
     if (!(ew <= ESDC_VTAB_TOL) || !(el <= ESDC_VTAB_TOL)) {
-        rows.clear();
+        rows.reset();
         return -2;
     }
     return 0;

@@ -179,7 +179,7 @@ struct Cached {
     int M;
     double dt;
     ColloData C;
-    std::vector<double> rows;
+    TableRows rows;
     double err;
 };
 std::mutex g_mu;
@@ -188,9 +188,9 @@ constexpr size_t kCacheSize = 8;
 
 }  // namespace
 
-int esdc_ztab_build(int M, double dt, const ColloData& C, std::vector<double>& rows, double* err_out)
+int esdc_ztab_build(int M, double dt, const ColloData& C, TableRows& rows, double* err_out)
 {
-    rows.clear();
+    rows.reset();
     if (M < 1 || M > ESDC_MMAX || !(dt > 0.0) || !std::isfinite(dt)) return -1;
     double err = 0.0;
     bool hit = false;
@@ -210,7 +210,7 @@ int esdc_ztab_build(int M, double dt, const ColloData& C, std::vector<double>& r
     }
     if (!hit) {
         const int nrow = ESDC_ZTAB_OCT << ESDC_ZTAB_SUB;
-        rows.assign((size_t)nrow * ESDC_ZTAB_ROW(M), 0.0);
+        std::vector<double> v((size_t)nrow * ESDC_ZTAB_ROW(M), 0.0);
         unsigned nt = std::thread::hardware_concurrency();
         nt = std::max(1u, std::min(nt, 16u));
         std::vector<double> te(nt, 0.0);
@@ -219,9 +219,10 @@ int esdc_ztab_build(int M, double dt, const ColloData& C, std::vector<double>& r
         for (unsigned t = 0; t < nt; ++t) {
             const int r0 = (int)t * per, r1 = std::min(nrow, r0 + per);
             if (r0 >= r1) break;
-            th.emplace_back(build_rows, M, std::cref(C), dt, r0, r1, rows.data(), std::ref(te[t]));
+            th.emplace_back(build_rows, M, std::cref(C), dt, r0, r1, v.data(), std::ref(te[t]));
         }
         for (auto& x : th) x.join();
+        rows = std::make_shared<const std::vector<double>>(std::move(v));
         for (double v : te) err = std::fmax(err, v);
         std::lock_guard<std::mutex> lk(g_mu);
         if (g_cache.size() >= kCacheSize) g_cache.erase(g_cache.begin());
@@ -229,7 +230,7 @@ int esdc_ztab_build(int M, double dt, const ColloData& C, std::vector<double>& r
     }
     if (err_out) *err_out = err;
     if (!(err <= ESDC_ZTAB_TOL)) {
-        rows.clear();
+        rows.reset();
         return -2;
     }
     return 0;
