@@ -45,6 +45,30 @@ __device__ __forceinline__ Q4<float> ld4(const float* a)
     return {{u.x, u.y, u.z, u.w}};
 }
 
+// FP32 value as FP64 by integer operations (the FP64 pipe also does the
+// conversions, at its own rate): exact for normal numbers and zero, FP32
+// subnormals become zero; not for Inf and NaN.
+__device__ __forceinline__ double widen(float f)
+{
+    const unsigned u = __float_as_uint(f), a = u & 0x7fffffffu;
+    const bool z = a < 0x00800000u;
+    return __hiloint2double((int)((u & 0x80000000u) | (z ? 0u : (a >> 3) + 0x38000000u)), z ? 0 : (int)(u << 29));
+}
+
+// A value, and a quad, of storage type S as type T.
+template <typename T, typename S> struct Load {
+    static __device__ __forceinline__ T one(const S* a) { return __ldcg(a); }
+    static __device__ __forceinline__ Q4<T> four(const S* a) { return ld4(a); }
+};
+template <> struct Load<double, float> {
+    static __device__ __forceinline__ double one(const float* a) { return widen(__ldcg(a)); }
+    static __device__ __forceinline__ Q4<double> four(const float* a)
+    {
+        const Q4<float> q = ld4(a);
+        return {{widen(q.v[0]), widen(q.v[1]), widen(q.v[2]), widen(q.v[3])}};
+    }
+};
+
 __device__ __forceinline__ void st4(double* a, const Q4<double>& q)
 {
     __stcg(reinterpret_cast<double2*>(a), make_double2(q.v[0], q.v[1]));
@@ -178,20 +202,21 @@ __device__ __forceinline__ DiagIdx diag_idx(const Geo& G)
     return d;
 }
 
-// out = (I - g A) v on the quad; c = v on the quad.
-template <typename T, bool LAY>
-__device__ __forceinline__ void apply4(const MeshDev& m, const Tab<T>& t, const T* v, const Geo& G,
+// out = (I - g A) v on the quad; c = v on the quad (v stored as S, arithmetic in T).
+template <typename T, bool LAY, typename S>
+__device__ __forceinline__ void apply4(const MeshDev& m, const Tab<T>& t, const S* v, const Geo& G,
                                        const DiagIdx& di, Q4<T>& c, Q4<T>& out)
 {
     const int nx = m.nx, sxy = m.nx * m.ny, p = G.p;
-    c = ld4(v + p);
-    const T vl = G.xl ? __ldcg(v + p - 1) : T(0);
-    const T vr = G.xr ? __ldcg(v + p + 4) : T(0);
+    using L = Load<T, S>;
+    c = L::four(v + p);
+    const T vl = G.xl ? L::one(v + p - 1) : T(0);
+    const T vr = G.xr ? L::one(v + p + 4) : T(0);
     Q4<T> vn = {{T(0), T(0), T(0), T(0)}}, vs = vn, vb = vn, vt = vn;
-    if (G.yn) vn = ld4(v + p - nx);
-    if (G.ys) vs = ld4(v + p + nx);
-    if (G.zb) vb = ld4(v + p - sxy);
-    if (G.zt) vt = ld4(v + p + sxy);
+    if (G.yn) vn = L::four(v + p - nx);
+    if (G.ys) vs = L::four(v + p + nx);
+    if (G.zb) vb = L::four(v + p - sxy);
+    if (G.zt) vt = L::four(v + p + sxy);
     const T dl = t.D[di.l], dm = t.D[di.m], dr = t.D[di.r];
     if (!LAY) {
 #pragma unroll
@@ -204,10 +229,10 @@ __device__ __forceinline__ void apply4(const MeshDev& m, const Tab<T>& t, const 
         }
     } else {
         // in-plane diagonal neighbours outside the quad's x range
-        const T nl = (G.xl && G.yn) ? __ldcg(v + p - nx - 1) : T(0);   // (x0-1, y-1)
-        const T nr = (G.xr && G.yn) ? __ldcg(v + p - nx + 4) : T(0);   // (x0+4, y-1)
-        const T sl = (G.xl && G.ys) ? __ldcg(v + p + nx - 1) : T(0);   // (x0-1, y+1)
-        const T sr = (G.xr && G.ys) ? __ldcg(v + p + nx + 4) : T(0);   // (x0+4, y+1)
+        const T nl = (G.xl && G.yn) ? L::one(v + p - nx - 1) : T(0);   // (x0-1, y-1)
+        const T nr = (G.xr && G.yn) ? L::one(v + p - nx + 4) : T(0);   // (x0+4, y-1)
+        const T sl = (G.xl && G.ys) ? L::one(v + p + nx - 1) : T(0);   // (x0-1, y+1)
+        const T sr = (G.xr && G.ys) ? L::one(v + p + nx + 4) : T(0);   // (x0+4, y+1)
         const T cx = t.cx[G.iz], cy = t.cy[G.iz], cd = t.cd[G.iz];
         const T czb = G.zb ? t.cz[G.iz - 1] : T(0), czt = t.cz[G.iz];
 #pragma unroll
@@ -378,71 +403,63 @@ __global__ void __launch_bounds__(ESDC_CG_THREADS) k_cg4(CgArgs a)
 // stencil's extra neighbours and coefficients need more registers: 512.
 template <bool LAY> constexpr int cheb_threads() { return LAY ? 512 : ESDC_CHEB_THREADS; }
 
-template <bool LAY>
-__global__ void __launch_bounds__(cheb_threads<LAY>(), 1) k_cheb4(CgArgs a, ChebArgs c)
+// The residual pass r = b - B x of the quads [q0, q1) with the partial sums of
+// r.r and b.b; d = r / theta (D64) or the FP32 copy of r (!D64).
+template <bool LAY, bool D64>
+__device__ __forceinline__ void cheb4_start(const CgArgs& a, const Tab<double>& t, int q0, int q1, double inv_theta,
+                                            double* d64, float* r32, double (&v)[2])
 {
-    extern __shared__ __align__(16) unsigned char dsm[];
     const MeshDev& m = a.m;
-    Tab<double> t = carve<double>(reinterpret_cast<double*>(dsm), m);
-    build_tab(m, a.g, false, t);
-    const int nq = m.N >> 2;
-    // a contiguous, balanced range of quads per block (one block per SM)
-    const int q0 = (int)((long long)blockIdx.x * nq / gridDim.x);
-    const int q1 = (int)((long long)(blockIdx.x + 1) * nq / gridDim.x);
+    for (int qi = q0 + (int)threadIdx.x; qi < q1; qi += blockDim.x) {
+        const Geo G = geo(m, qi);
+        const DiagIdx di = diag_idx<LAY>(G);
+        Q4<double> xc, bx;
+        apply4<double, LAY>(m, t, a.x, G, di, xc, bx);
+        const Q4<double> b = ld4(a.b + G.p);
+        Q4<double> r, d;
+        Q4<float> rf;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            r.v[j] = b.v[j] - bx.v[j];
+            if (D64) d.v[j] = r.v[j] * inv_theta;
+            else rf.v[j] = (float)r.v[j];
+            v[0] = fma(r.v[j], r.v[j], v[0]);
+            v[1] = fma(b.v[j], b.v[j], v[1]);
+        }
+        st4(a.r + G.p, r);
+        if (D64) st4(d64 + G.p, d);
+        else st4(r32 + G.p, rf);
+    }
+}
+
+// The iterations of the semi-iteration from r (a.r, norm^2 rr) and d_0 = r / theta
+// (a.p) until r.r <= stop, a non-finite residual or the cap; false: a wait ran out.
+template <bool LAY>
+__device__ bool cheb4_iterate(const CgArgs& a, const ChebArgs& c, const Tab<double>& t, int q0, int q1, double rr0,
+                              double stop, unsigned& target, int& it, bool& done, bool& bad)
+{
+    const MeshDev& m = a.m;
     double* part = a.part;
-    __shared__ double bs[3];
-    unsigned target = 0;
     double* dc = a.p;            // d_k
     double* dn = a.q;            // d_{k+1}
-    const double inv_theta = c.inv_theta;
-
-    // r = b - B x, d_0 = r / theta; partials r.r, b.b
-    {
-        double v[2] = {0.0, 0.0};
-        for (int qi = q0 + (int)threadIdx.x; qi < q1; qi += blockDim.x) {
-            const Geo G = geo(m, qi);
-            const DiagIdx di = diag_idx<LAY>(G);
-            Q4<double> xc, bx;
-            apply4<double, LAY>(m, t, a.x, G, di, xc, bx);
-            const Q4<double> b = ld4(a.b + G.p);
-            Q4<double> r, d;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                r.v[j] = b.v[j] - bx.v[j];
-                d.v[j] = r.v[j] * inv_theta;
-                v[0] = fma(r.v[j], r.v[j], v[0]);
-                v[1] = fma(b.v[j], b.v[j], v[1]);
-            }
-            st4(a.r + G.p, r);
-            st4(dc + G.p, d);
-        }
-        block_sum<2>(v, bs);
-        if (threadIdx.x == 0) for (int k = 0; k < 2; ++k) part[k * gridDim.x + blockIdx.x] = bs[k];
-    }
-    if (!grid_barrier(a.bar, target, a.flags)) return;
-    double tot[2];
-    grid_total<2>(part, 0, tot);
-    const double stop = a.tol2 * tot[1];
-    bool done = tot[0] <= stop;
-    bool bad = !isfinite(tot[0]) || !isfinite(stop);
+    __shared__ double bs[1];
     // iterations the bound asks for: 2 q^k ||r_0|| <= tol ||b||.  One thread per block
     // evaluates it (a few dozen FP64 operations) and shares it; every block gets the same value.
     __shared__ int s_kneed;
     if (threadIdx.x == 0) {
         int kn = 1;
         if (!done && !bad && c.q > 0.0) {
-            const double kd = stop > 0.0 ? ceil(log(0.5 * sqrt(stop / tot[0])) / c.log_q) : (double)a.maxit;
+            const double kd = stop > 0.0 ? ceil(log(0.5 * sqrt(stop / rr0)) / c.log_q) : (double)a.maxit;
             kn = kd < (double)a.maxit ? (int)kd : a.maxit;     // tol 0: run to the cap
         }
         s_kneed = kn < 1 ? 1 : kn;
     }
     __syncthreads();
-    const int k_need = s_kneed;
-    int it = 0;
-    int chunk_end = k_need < a.maxit ? k_need : a.maxit;
+    const int it0 = it;
+    int chunk_end = it0 + s_kneed < a.maxit ? it0 + s_kneed : a.maxit;
     while (!done && !bad && it < a.maxit) {
         const bool check = it + 1 >= chunk_end;
-        const int ki = it < ESDC_CHEB_TAB ? it : ESDC_CHEB_TAB - 1;
+        const int k = it - it0, ki = k < ESDC_CHEB_TAB ? k : ESDC_CHEB_TAB - 1;
         const double ca = c.ca[ki], cb = c.cb[ki];
         double v[1] = {0.0};
         for (int qi = q0 + (int)threadIdx.x; qi < q1; qi += blockDim.x) {
@@ -469,7 +486,7 @@ __global__ void __launch_bounds__(cheb_threads<LAY>(), 1) k_cheb4(CgArgs a, Cheb
             block_sum<1>(v, bs);
             if (threadIdx.x == 0) part[(2 + (it & 1)) * gridDim.x + blockIdx.x] = bs[0];
         }
-        if (!grid_barrier(a.bar, target, a.flags)) return;
+        if (!grid_barrier(a.bar, target, a.flags)) return false;
         if (check) {
             double rr[1];
             grid_total<1>(part, 2 + (it & 1), rr);
@@ -478,12 +495,230 @@ __global__ void __launch_bounds__(cheb_threads<LAY>(), 1) k_cheb4(CgArgs a, Cheb
             chunk_end = it + 2 < a.maxit ? it + 2 : a.maxit;     // rounding left it short: two more, then check
         }
     }
+    return true;
+}
+
+__device__ __forceinline__ void cheb4_report(const CgArgs& a, int it, bool done, bool bad)
+{
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         a.status[0] = it;
         if (a.iter_log) *a.iter_log = it;
         if (bad) atomicOr(a.flags, ESDC_FLAG_NONFINITE);
         else if (!done) atomicOr(a.flags, ESDC_FLAG_CG_MAXIT);
     }
+}
+
+template <bool LAY>
+__global__ void __launch_bounds__(cheb_threads<LAY>(), 1) k_cheb4(CgArgs a, ChebArgs c)
+{
+    extern __shared__ __align__(16) unsigned char dsm[];
+    const MeshDev& m = a.m;
+    Tab<double> t = carve<double>(reinterpret_cast<double*>(dsm), m);
+    build_tab(m, a.g, false, t);
+    const int nq = m.N >> 2;
+    // a contiguous, balanced range of quads per block (one block per SM)
+    const int q0 = (int)((long long)blockIdx.x * nq / gridDim.x);
+    const int q1 = (int)((long long)(blockIdx.x + 1) * nq / gridDim.x);
+    __shared__ double bs[2];
+    unsigned target = 0;
+    double v[2] = {0.0, 0.0};
+    cheb4_start<LAY, true>(a, t, q0, q1, c.inv_theta, a.p, nullptr, v);
+    block_sum<2>(v, bs);
+    if (threadIdx.x == 0) for (int k = 0; k < 2; ++k) a.part[k * gridDim.x + blockIdx.x] = bs[k];
+    if (!grid_barrier(a.bar, target, a.flags)) return;
+    double tot[2];
+    grid_total<2>(a.part, 0, tot);
+    const double stop = a.tol2 * tot[1];
+    bool done = tot[0] <= stop;
+    bool bad = !isfinite(tot[0]) || !isfinite(stop);
+    int it = 0;
+    if (!cheb4_iterate<LAY>(a, c, t, q0, q1, tot[0], stop, target, it, done, bad)) return;
+    cheb4_report(a, it, done, bad);
+}
+
+// The same solve to the same stop test with the iterations in FP32: corrections
+// e of (I - g A) e = r by Chebyshev iterations on FP32 vectors, each then taken
+// off the FP64 residual (r -= B e in FP64, e widened exactly) and added to x in
+// FP64.  An FP64 iteration of a large mesh costs its 13 (scalar) to 19 (layered)
+// FP64-pipe operations per node: 110 us at 4.2M nodes where its bytes take 30.
+// The FP32 iteration moves 24 bytes per node and leaves the FP64 pipe alone:
+// 1293 -> 530 us per solve of the 256x256x64 layered slab, and from 305,000 to 350,000
+// nodes on it is the faster one (600x500 scalar sheet 2.21 / 2.19 ms per step,
+// 128x128x64 layered slab 7.32 / 5.35; 300x250 sheet 0.97 / 1.28, barrier-bound).
+//
+// A correction reduces the residual by 3e-6 at most (FP32 rounding leaves about
+// kappa 6e-8) and the passes share the reduction that the stop test needs, so a
+// warm-started solve takes two.  The last correction's own FP32 residual tells
+// whether it met the test, with 2e-6 ||r|| (the residual it started from) as the
+// allowance for its rounding; else the FP64 residual decides and the passes go
+// on.  What refinement cannot do (residuals near FP32's range, no progress) the
+// FP64 iterations finish.  The result has FP64's error: every correction but the
+// last is measured by an FP64 residual, and the last one's rounding (1e-7 of a
+// correction of 1e-9 and below) is under x's own.
+struct RefArgs {
+    float *r, *z, *p, *q, *e;
+    double qq[ESDC_CHEB_TAB];       // 4 q^{2 (k + 1)}
+    double fmin2;                   // least reduction (squared) asked of one correction
+};
+#define ESDC_REF_MAXOUT 8
+
+template <bool LAY>
+__global__ void __launch_bounds__(cheb_threads<LAY>(), 1) k_cheb4_ref(CgArgs a, ChebArgs c, RefArgs f)
+{
+    extern __shared__ __align__(16) unsigned char dsm[];
+    const MeshDev& m = a.m;
+    const int ne = tab_entries(m);
+    Tab<double> t = carve<double>(reinterpret_cast<double*>(dsm), m);
+    Tab<float> tf = carve<float>(reinterpret_cast<float*>(dsm + sizeof(double) * ne), m);
+    build_tab(m, a.g, false, t);
+    build_tab(m, a.g, false, tf);
+    const int nq = m.N >> 2;
+    const int q0 = (int)((long long)blockIdx.x * nq / gridDim.x);
+    const int q1 = (int)((long long)(blockIdx.x + 1) * nq / gridDim.x);
+    double* part = a.part;
+    __shared__ double bs[2];
+    __shared__ int s_kin;
+    unsigned target = 0;
+    const float inv_theta = (float)c.inv_theta;
+    {
+        double v[2] = {0.0, 0.0};
+        cheb4_start<LAY, false>(a, t, q0, q1, 0.0, nullptr, f.r, v);
+        block_sum<2>(v, bs);
+        if (threadIdx.x == 0) for (int k = 0; k < 2; ++k) part[k * gridDim.x + blockIdx.x] = bs[k];
+    }
+    if (!grid_barrier(a.bar, target, a.flags)) return;
+    double tot[2];
+    grid_total<2>(part, 0, tot);
+    double rr = tot[0];
+    const double stop = a.tol2 * tot[1];
+    bool done = rr <= stop;
+    bool bad = !isfinite(rr) || !isfinite(stop);
+    int it = 0;
+    // FP32's range: the squares of a residual of rms 1e-13 to 1e13, reduced by 3e-6, stay in it
+    bool fp32 = rr > 1e-26 * m.N && rr < 1e26 * m.N;
+    for (int outer = 0; !done && !bad && fp32 && outer < ESDC_REF_MAXOUT && it < a.maxit; ++outer) {
+        // this correction's share of the reduction to a tenth of the stop test (what FP64
+        // iterations to the bound reach): all of it if one correction can, else the square
+        // root of what is left
+        const double f2 = 0.01 * stop / rr;
+        const bool final = f2 >= f.fmin2;
+        if (threadIdx.x < 32) {
+            const double want = final ? f2 : fmax(sqrt(f2), f.fmin2);
+            int kin = ESDC_CHEB_TAB;
+            for (int k0 = 0; k0 < ESDC_CHEB_TAB; k0 += 32) {
+                const unsigned hit = __ballot_sync(0xffffffffu, f.qq[k0 + threadIdx.x] <= want);
+                if (hit) { kin = k0 + __ffs(hit); break; }
+            }
+            if (threadIdx.x == 0) s_kin = kin;
+        }
+        __syncthreads();
+        const int kin = it + s_kin < a.maxit ? s_kin : a.maxit - it;
+        // e += d, r -= B d, d = ca d + cb r from e = 0, d = r / theta
+        float* dc = f.p;
+        float* dn = f.q;
+        double v[1] = {0.0};
+        for (int k = 0; k < kin; ++k) {
+            const int ki = k < ESDC_CHEB_TAB ? k : ESDC_CHEB_TAB - 1;
+            const float ca = (float)c.ca[ki], cb = (float)c.cb[ki];
+            const bool last = k + 1 == kin;
+            float acc = 0.0f;
+            for (int qi = q0 + (int)threadIdx.x; qi < q1; qi += blockDim.x) {
+                const Geo G = geo(m, qi);
+                const DiagIdx di = diag_idx<LAY>(G);
+                Q4<float> d, bd, ev, rv, en, rn, dnew;
+                if (k == 0) {
+                    apply4<float, LAY>(m, tf, f.r, G, di, rv, bd);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        d.v[j] = rv.v[j] * inv_theta;
+                        bd.v[j] *= inv_theta;
+                        ev.v[j] = 0.0f;
+                    }
+                } else {
+                    apply4<float, LAY>(m, tf, dc, G, di, d, bd);
+                    ev = ld4(f.e + G.p);
+                    rv = ld4(f.z + G.p);
+                }
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    en.v[j] = ev.v[j] + d.v[j];
+                    rn.v[j] = rv.v[j] - bd.v[j];
+                    dnew.v[j] = fmaf(ca, d.v[j], cb * rn.v[j]);
+                }
+                st4(f.e + G.p, en);
+                if (!last) {
+                    st4(f.z + G.p, rn);
+                    st4(dn + G.p, dnew);
+                } else {
+                    // in FP32's range: see fp32
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) acc = fmaf(rn.v[j], rn.v[j], acc);
+                }
+            }
+            v[0] += acc;
+            float* sw = dc; dc = dn; dn = sw;
+            if (last) {
+                block_sum<1>(v, bs);
+                if (threadIdx.x == 0) part[(4 + (outer & 1)) * gridDim.x + blockIdx.x] = bs[0];
+            }
+            if (!grid_barrier(a.bar, target, a.flags)) return;
+        }
+        it += kin;
+        double r32[1];
+        grid_total<1>(part, 4 + (outer & 1), r32);
+        if (!isfinite(r32[0])) { fp32 = false; break; }        // x and a.r are untouched: FP64 from here
+        if (final && sqrt(r32[0]) + 2e-6 * sqrt(rr) <= sqrt(stop)) {
+            for (int qi = q0 + (int)threadIdx.x; qi < q1; qi += blockDim.x) {
+                const Q4<float> e = ld4(f.e + 4 * qi);
+                Q4<double> x = ld4(a.x + 4 * qi);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) x.v[j] += widen(e.v[j]);
+                st4(a.x + 4 * qi, x);
+            }
+            done = true;
+            break;
+        }
+        // r -= B e, x += e in FP64
+        double w[1] = {0.0};
+        for (int qi = q0 + (int)threadIdx.x; qi < q1; qi += blockDim.x) {
+            const Geo G = geo(m, qi);
+            const DiagIdx di = diag_idx<LAY>(G);
+            Q4<double> e, be;
+            apply4<double, LAY>(m, t, f.e, G, di, e, be);
+            Q4<double> r = ld4(a.r + G.p), x = ld4(a.x + G.p);
+            Q4<float> rf;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                r.v[j] -= be.v[j];
+                x.v[j] += e.v[j];
+                rf.v[j] = (float)r.v[j];
+                w[0] = fma(r.v[j], r.v[j], w[0]);
+            }
+            st4(a.r + G.p, r);
+            st4(a.x + G.p, x);
+            st4(f.r + G.p, rf);
+        }
+        block_sum<1>(w, bs);
+        if (threadIdx.x == 0) part[(6 + (outer & 1)) * gridDim.x + blockIdx.x] = bs[0];
+        if (!grid_barrier(a.bar, target, a.flags)) return;
+        double rn[1];
+        grid_total<1>(part, 6 + (outer & 1), rn);
+        bad = !isfinite(rn[0]);
+        done = rn[0] <= stop;
+        fp32 = rn[0] <= 1e-2 * rr && rn[0] > 1e-26 * m.N;      // no progress: FP64 from here
+        rr = rn[0];
+    }
+    if (!done && !bad && it < a.maxit) {
+        for (int qi = q0 + (int)threadIdx.x; qi < q1; qi += blockDim.x) {
+            Q4<double> d = ld4(a.r + 4 * qi);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) d.v[j] *= c.inv_theta;
+            st4(a.p + 4 * qi, d);
+        }
+        if (!grid_barrier(a.bar, target, a.flags)) return;
+        if (!cheb4_iterate<LAY>(a, c, t, q0, q1, rr, stop, target, it, done, bad)) return;
+    }
+    cheb4_report(a, it, done, bad);
 }
 
 // ---------------------------------------------------------------- iterative refinement
@@ -882,24 +1117,33 @@ cudaError_t esdc_cheb_launch(const CgArgsHost& h, cudaStream_t s)
     ChebArgs c;
     if (!esdc_cheb_interval(h.mesh, h.g, c)) return esdc_cg4_launch(h, false, s);    // no interval
     const int ne = tab_entries(h.mesh);
-    const size_t bytes = sizeof(double) * ne;
     const bool lay = h.mesh.lay != nullptr;
-    cudaError_t e = lay ? prepare(k_cheb4<true>, bytes) : prepare(k_cheb4<false>, bytes);
+    // The FP32 corrections where the FP64 pipe bounds an iteration (larger meshes) and FP32
+    // can reduce a residual by 3e-6 (q at most 7/9, kappa at most 64).
+    const bool ref = h.w.r32 && h.mesh.N >= ESDC_REF_MIN_NODES && c.q > 0.0 && c.q < 7.0 / 9.0;
+    const size_t bytes = (sizeof(double) + (ref ? sizeof(float) : 0)) * ne;
+    const void* k = ref ? (lay ? (const void*)k_cheb4_ref<true> : (const void*)k_cheb4_ref<false>)
+                        : (lay ? (const void*)k_cheb4<true> : (const void*)k_cheb4<false>);
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
     if (e != cudaSuccess) return e;
     // One block per SM, balanced ranges of quads (blocks of at least 128 quads on small meshes).
     int threads = lay ? cheb_threads<true>() : cheb_threads<false>(), per_sm = 0;
-    if ((e = lay ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cheb4<true>, threads, bytes)
-                 : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_cheb4<false>, threads, bytes)) !=
-        cudaSuccess)
-        return e;
+    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, threads, bytes)) != cudaSuccess) return e;
     if (per_sm < 1) threads = h.w.threads;              // fewer registers than expected: the CG block size
     const long long nq = h.mesh.N / 4;
     long long nb = (nq + 127) / 128;
     if (nb > h.w.max_blocks) nb = h.w.max_blocks;
     if (nb < 1) nb = 1;
     if ((e = cudaMemsetAsync(h.w.bar, 0, sizeof(unsigned), s)) != cudaSuccess) return e;
-    void* args[] = {&a, &c};
-    const void* k = lay ? (const void*)k_cheb4<true> : (const void*)k_cheb4<false>;
+    RefArgs f;
+    f.r = h.w.r32; f.z = h.w.z32; f.p = h.w.p32; f.q = h.w.q32; f.e = h.w.e32;
+    f.fmin2 = 1e-11;
+    double q2 = 1.0;
+    for (int i = 0; i < ESDC_CHEB_TAB; ++i) {
+        q2 *= c.q * c.q;
+        f.qq[i] = 4.0 * q2;
+    }
+    void* args[] = {&a, &c, &f};
     return cudaLaunchCooperativeKernel(k, dim3((unsigned)nb), dim3(threads), args, bytes, s);
 }
 

@@ -166,10 +166,16 @@ struct SmallDev {
     int mat_doubles = 0;
 };
 
+// Mesh size from which the FP64 Chebyshev solves iterate on FP32 corrections.
+#ifndef ESDC_REF_MIN_NODES
+#define ESDC_REF_MIN_NODES 400000
+#endif
 // CG solve on the handle's mesh: (I - g L) x = b (Jacobi-preconditioned).
 struct CgWork {
     double *r, *p, *q, *z;          // [ld] each
-    float *r32, *p32, *q32, *z32, *e32;   // [ld] each, precision form only (else null)
+    // [ld] each: the precision form's, and on the FP64 path those of the FP32 corrections
+    // (meshes of at least ESDC_REF_MIN_NODES nodes with Chebyshev solves); else null
+    float *r32, *p32, *q32, *z32, *e32;
     double* part;                   // [8 * max_blocks] block partial sums
     unsigned* bar;                  // [4] grid barrier: arrival count, spare, and two test words (grid_barrier)
     int* status;                    // [2]: iterations of the last solve, flag bits

@@ -404,7 +404,8 @@ int esdc_create(const esdc_mesh* mesh, double sigma, double chi, double Cm, int 
         h->cg_log = reinterpret_cast<int*>(c + rmax_b + flag_b);
         h->cg.bar = reinterpret_cast<unsigned*>(c + rmax_b + flag_b + log_b);
     }
-    if (o.precision == 1) {                       // FP32 vectors of the inner solves
+    // FP32 vectors: the precision form's inner solves, the FP64 solves' corrections
+    if (o.precision == 1 || ((o.solver == 0 || o.solver == 3) && h->mesh.N >= ESDC_REF_MIN_NODES)) {
         float** fv[] = {&h->cg.r32, &h->cg.p32, &h->cg.q32, &h->cg.z32, &h->cg.e32};
         for (float** f : fv) {
             if (cudaMalloc((void**)f, sizeof(float) * ld) != cudaSuccess) return fail(ESDC_ERR_NO_MEMORY);
