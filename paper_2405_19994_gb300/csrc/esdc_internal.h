@@ -80,22 +80,16 @@ struct StimDev {
     double amp[ESDC_MAXBOX], t_on[ESDC_MAXBOX], t_off[ESDC_MAXBOX];
 };
 
-// The gate functions tabulated in V (esdc_vtab.cpp; SYN19 and HH1952): ESDC_VTAB_N
-// intervals of ESDC_VTAB_W mV from ESDC_VTAB_VLO, a polynomial of degree
-// ESDC_VTAB_NC - 1 in t = V - V_mid per function and interval; a row holds
-// V_mid and a pad (16-byte alignment), then per gate the coefficient pairs
-// (b, Lambda) of t^0, t^1, ..., b = -Lambda w_inf, so that one 16-byte load feeds both
-// Horner recurrences.
+// The gate functions tabulated in V (esdc_vtab.cpp; SYN19 and HH1952):
+// ESDC_VTAB_N intervals of ESDC_VTAB_W mV centred at ESDC_VTAB_VLO + i ESDC_VTAB_W,
+// a cubic in t = V - centre per function and interval (esdc_tabeval.h); a row
+// holds per gate the cubics of b = -Lambda w_inf and of Lambda.
 #define ESDC_VTAB_VLO (-140.0)
-#ifndef ESDC_VTAB_W
-#define ESDC_VTAB_W 0.0078125      // interval width (mV): 1/128, a power of two
-#endif
-#ifndef ESDC_VTAB_NC
-#define ESDC_VTAB_NC 4             // coefficients per function (degree 3)
-#endif
-#define ESDC_VTAB_N ((int)(240.0 / ESDC_VTAB_W))
-#define ESDC_VTAB_ROW (2 + 2 * ESDC_NGMAX * ESDC_VTAB_NC)
-#define ESDC_VTAB_TOL 4e-15        // refuse a table whose FP64 evaluation misses by more
+#define ESDC_VTAB_LGW 7            // interval width 2^-7 mV
+#define ESDC_VTAB_W 0.0078125
+#define ESDC_VTAB_N (240 * 128 + 1)
+#define ESDC_VTAB_ROW (2 * 4 * ESDC_NGMAX)   // doubles per row: two 32-byte cubics per gate
+#define ESDC_VTAB_TOL 4e-15        // refuse a table whose evaluation misses by more
 struct ModelDev {
     double p[ESDC_NPMAX];
     const double* vtab = nullptr;  // the gate table, or nullptr: direct evaluation
@@ -206,25 +200,19 @@ cudaError_t esdc_dct_launch(const MeshDev& m, const CgWork& w, double g, const d
 // A table's rows, shared with the process's cache of built tables.
 using TableRows = std::shared_ptr<const std::vector<double>>;
 // The gate table of a model (SYN19, HH1952): rows [ESDC_VTAB_N][ESDC_VTAB_ROW] and
-// the largest errors of its FP64 evaluation against the direct functions
+// the largest errors of its evaluation against the direct functions
 // (absolute for w_inf, relative for Lambda).  0: built; -1: no table for this
 // model; -2: an error above ESDC_VTAB_TOL (no rows).
 int esdc_vtab_build(int model, const double* params, TableRows& rows, double* err_winf, double* err_lam);
 
 // The set-up's exponential coefficients tabulated in y = 1 - z, z = dt Lambda
-// (esdc_ztab.cpp): ESDC_ZTAB_OCT octaves of y, 2^ESDC_ZTAB_SUB intervals each,
-// a polynomial of degree ESDC_ZTAB_NC - 1 per function and interval; a row
-// holds y_mid, a pad, then for i = 0..M-1 the coefficients of dt d_{i+1}
-// phi_1(d_{i+1} z) and of dt S_{i+1,j}(z), j = 0..M-1.
+// (esdc_ztab.cpp): ESDC_ZTAB_OCT octaves of y, 2^ESDC_ZTAB_SUB intervals each, a
+// cubic per function and interval (esdc_tabeval.h); a row holds, for i = 0..M-1,
+// dt d_{i+1} phi_1(d_{i+1} z) and dt S_{i+1,j}(z), j = 0..M-1.
 #define ESDC_ZTAB_OCT 12
-#ifndef ESDC_ZTAB_SUB
 #define ESDC_ZTAB_SUB 10           // 1024 intervals per octave of y
-#endif
-#ifndef ESDC_ZTAB_NC
-#define ESDC_ZTAB_NC 4             // coefficients per function (degree 3)
-#endif
-#define ESDC_ZTAB_ROW(M) (2 + (M) * ((M) + 1) * ESDC_ZTAB_NC)
-#define ESDC_ZTAB_TOL 4e-15         // refuse a table whose FP64 evaluation misses by more (units of dt)
+#define ESDC_ZTAB_ROW(M) ((M) * ((M) + 1) * 4)   // doubles per row: 32-byte cubics
+#define ESDC_ZTAB_TOL 4e-15         // refuse a table whose evaluation misses by more (units of dt)
 // Builds (or takes from this process's cache) the table for (M, dt, C);
 // returns 0, -1 (bad arguments) or -2 (error above ESDC_ZTAB_TOL, no
 // rows); *err: the largest error, in units of dt.

@@ -190,16 +190,6 @@ struct PhaseArgs {
 };
 __device__ __forceinline__ PhaseArgs phase_of(const StepArgs& a) { return PhaseArgs{a.i, a.rho, a.Gold, a.Gnew, a.yout}; }
 
-// One function of the set-up table (esdc_ztab.cpp) at t: Horner's rule on its
-// ESDC_ZTAB_NC coefficients.
-__device__ __forceinline__ double ztab_poly(const double* __restrict__ c, double t)
-{
-    double r = __ldg(c + ESDC_ZTAB_NC - 1);
-#pragma unroll
-    for (int k = ESDC_ZTAB_NC - 2; k >= 0; --k) r = fma(r, t, __ldg(c + k));
-    return r;
-}
-
 // Per-step tables of gate g at node p: Lambda_n, dt d_i phi_1(d_i dt Lambda_n)
 // and dt S_ij(dt Lambda_n) (App. A).  From the set-up table when there is one
 // and z = dt Lambda_n lies in its range (1 <= y = 1 - z < 2^ESDC_ZTAB_OCT: the
@@ -217,16 +207,19 @@ __device__ __forceinline__ void gate_tables(const StepArgs& a, int g, int NG, do
         const int e = (int)(bits >> 52) - 1023;             // NaN, Inf and y < 1 fall outside
         if (e >= 0 && e < ESDC_ZTAB_OCT) {
             const int r = (e << ESDC_ZTAB_SUB) + (int)((bits >> (52 - ESDC_ZTAB_SUB)) & ((1 << ESDC_ZTAB_SUB) - 1));
-            const double* row = a.ztab + (size_t)r * ESDC_ZTAB_ROW(M);
-            const double t = y - __ldg(row);
-            const double* c = row + 2;
+            // the interval's middle: y's leading bits, and a one below them
+            const long long top = ~((1LL << (52 - ESDC_ZTAB_SUB)) - 1);
+            const double mid = __longlong_as_double((bits & top) | (1LL << (51 - ESDC_ZTAB_SUB)));
+            float th, tl;
+            esdc::tab_split(y - mid, th, tl);
+            const int4* c = reinterpret_cast<const int4*>(a.ztab + (size_t)r * ESDC_ZTAB_ROW(M));
 #pragma unroll
             for (int i = 0; i < M; ++i) {
-                a.PHI[((int64_t)i * NG + g) * ld + p] = ztab_poly(c + (i * (M + 1)) * ESDC_ZTAB_NC, t);
+                a.PHI[((int64_t)i * NG + g) * ld + p] = esdc::tab_at(c + 2 * (i * (M + 1)), th, tl);
 #pragma unroll
                 for (int j = 0; j < M; ++j)
                     a.S[(((int64_t)i * M + j) * NG + g) * ld + p] =
-                        ztab_poly(c + (i * (M + 1) + 1 + j) * ESDC_ZTAB_NC, t);
+                        esdc::tab_at(c + 2 * (i * (M + 1) + 1 + j), th, tl);
             }
             return;
         }

@@ -11,23 +11,49 @@
 #pragma once
 #include "esdc_fmath.cuh"
 #include "esdc_internal.h"
+#include "esdc_tabeval.h"
 
 namespace esdc {
 
-// The two polynomials of one gate in the gate table (esdc_vtab.cpp) at
-// t = V - V_mid: Horner's rule, ESDC_VTAB_NC - 1 FMAs each, on the interleaved
-// coefficient pairs c[k] = (b, Lambda) of t^k, b = -Lambda w_inf.
-__device__ __forceinline__ void vt_poly2(const double2* __restrict__ c, double t, double& w, double& l)
+// A table's cubic (two 16-byte loads) at t = th + tl.
+__device__ __forceinline__ double tab_at(const int4* __restrict__ c, float th, float tl)
 {
-    const double2 top = __ldg(c + ESDC_VTAB_NC - 1);
-    w = top.x;
-    l = top.y;
-#pragma unroll
-    for (int k = ESDC_VTAB_NC - 2; k >= 0; --k) {
-        const double2 ck = __ldg(c + k);
-        w = fma(w, t, ck.x);
-        l = fma(l, t, ck.y);
+    const int4 u = __ldg(c), v = __ldg(c + 1);
+    TabPoly p;
+    p.c0 = (int64_t)(((uint64_t)(uint32_t)u.y << 32) | (uint32_t)u.x);
+    p.c1h = __int_as_float(u.z);
+    p.c1l = __int_as_float(u.w);
+    p.c2h = __int_as_float(v.x);
+    p.c2l = __int_as_float(v.y);
+    p.c3 = __int_as_float(v.z);
+    p.eS = v.w;
+    return tab_eval(p, th, tl);
+}
+
+// The gate table at potential V: the row of the interval and t = V - centre, once
+// per node for all gates; row = nullptr (no table, or V outside it): the direct
+// formulas.  V + 1.5 2^(52 - ESDC_VTAB_LGW) rounds V to a multiple of the width and
+// holds the multiple in its low word; the high word is that of the constant for
+// every V in reach (not for NaN, Inf or large V).  Three FP64 additions.
+struct GateCtx {
+    const int4* row;
+    float th, tl;
+};
+__device__ __forceinline__ GateCtx gate_ctx(const ModelDev& md, double V)
+{
+    GateCtx c{nullptr, 0.0f, 0.0f};
+    if (md.vtab) {
+        constexpr double magic = 1.5 * (double)(1ULL << (52 - ESDC_VTAB_LGW));
+        const double s = V + magic;
+        const int i = __double2loint(s) - (int)(ESDC_VTAB_VLO * (1 << ESDC_VTAB_LGW));
+        const int top = __double2hiint(s);
+        const int want = __double2hiint(magic) - (__double2loint(s) < 0 ? 1 : 0);
+        if (top == want && i >= 0 && i < ESDC_VTAB_N) {
+            c.row = reinterpret_cast<const int4*>(md.vtab + (size_t)i * ESDC_VTAB_ROW);
+            tab_split(V - (s - magic), c.th, c.tl);
+        }
     }
+    return c;
 }
 
 // x/(e^x - 1), removable singularity at x = 0.  |x| < 1/2: its Taylor series
@@ -99,31 +125,17 @@ struct HH1952 {
         lam = -sum;
         yinf = al * esdc_rcp(sum);
     }
-    // The gate table (esdc_vtab.cpp), as for SYN19: the node's interval row
-    // and t = V - V_mid once per node; row = nullptr: the direct rates.
-    struct VCtx {
-        const double* row;
-        double t;
-    };
-    __device__ static VCtx vctx(const ModelDev& md, double V)
-    {
-        VCtx c{nullptr, 0.0};
-        if (md.vtab) {
-            const int i = __double2int_rd((V - ESDC_VTAB_VLO) * (1.0 / ESDC_VTAB_W));
-            if (i >= 0 && i < ESDC_VTAB_N) {
-                c.row = md.vtab + (size_t)i * ESDC_VTAB_ROW;
-                c.t = V - __ldg(c.row);
-            }
-        }
-        return c;
-    }
+    // The gate table (esdc_vtab.cpp): the node's interval once per node.
+    using VCtx = GateCtx;
+    __device__ static VCtx vctx(const ModelDev& md, double V) { return gate_ctx(md, V); }
     // Lambda_q and b_q = -Lambda_q w_inf,q (here alpha_q): the table, else the
     // direct rates.  The gate's rate is then Lambda u + b.
     __device__ static void gate_lb(const double* __restrict__ mp, const VCtx& c, int q, double V, double& lam,
                                    double& b)
     {
         if (c.row) {
-            vt_poly2(reinterpret_cast<const double2*>(c.row + 2) + q * ESDC_VTAB_NC, c.t, b, lam);
+            b = tab_at(c.row + 4 * q, c.th, c.tl);
+            lam = tab_at(c.row + 4 * q + 2, c.th, c.tl);
             return;
         }
         double yinf;
@@ -293,34 +305,17 @@ struct SYN19 {
         const double s = esdc_rcp(1.0 + esdc_exp(fma(-V, inv[12 + q], dv[12 + q])));
         lam = -esdc_exp(fma(p[3], s, dv[24 + q]));
     }
-    // The gate table (esdc_vtab.cpp): a node's interval row and t = V - V_mid,
-    // computed once per node for all twelve gates; row = nullptr (no table, or
-    // V outside [ESDC_VTAB_VLO, ESDC_VTAB_VLO + ESDC_VTAB_N ESDC_VTAB_W)) selects
-    // the direct evaluation.  A NaN V stays NaN either way.
-    struct VCtx {
-        const double* row;
-        double t;
-    };
-    __device__ static VCtx vctx(const ModelDev& md, double V)
-    {
-        VCtx c{nullptr, 0.0};
-        if (md.vtab) {
-            const int i = __double2int_rd((V - ESDC_VTAB_VLO) * (1.0 / ESDC_VTAB_W));
-            if (i >= 0 && i < ESDC_VTAB_N) {
-                c.row = md.vtab + (size_t)i * ESDC_VTAB_ROW;
-                c.t = V - __ldg(c.row);
-            }
-        }
-        return c;
-    }
-    // Lambda_q and b_q = -Lambda_q w_inf,q of gate q: two polynomials
-    // (2 (ESDC_VTAB_NC - 1) FMAs) on the table, else the direct formulas (about
-    // 35 FP64 operations).  The gate's rate is then Lambda u + b.
+    // The gate table (esdc_vtab.cpp): the node's interval once for all twelve gates.
+    using VCtx = GateCtx;
+    __device__ static VCtx vctx(const ModelDev& md, double V) { return gate_ctx(md, V); }
+    // Lambda_q and b_q = -Lambda_q w_inf,q of gate q: two cubics (no FP64 operation)
+    // on the table, else the direct formulas (about 35 FP64 operations).  The gate's rate is then Lambda u + b.
     __device__ static void gate_lb(const double* __restrict__ mp, const VCtx& c, int q, double V, double& lam,
                                    double& b)
     {
         if (c.row) {
-            vt_poly2(reinterpret_cast<const double2*>(c.row + 2) + q * ESDC_VTAB_NC, c.t, b, lam);
+            b = tab_at(c.row + 4 * q, c.th, c.tl);
+            lam = tab_at(c.row + 4 * q + 2, c.th, c.tl);
             return;
         }
         double yinf;

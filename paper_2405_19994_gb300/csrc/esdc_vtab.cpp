@@ -9,29 +9,23 @@
 // Evaluated directly a SYN19 gate costs three exponentials and two
 // reciprocals (about 35 FP64 operations), an HH gate about as much; on a GPU
 // with two FP64 lane operations per SM and clock that is most of the node
-// kernel.  Here each function is replaced, on each interval
-// [V_lo + i w, V_lo + (i+1) w) of width w = ESDC_VTAB_W (1/128 mV), by its
-// Chebyshev interpolant of degree ESDC_VTAB_NC - 1 (3: 4 Chebyshev points,
-// values in long double), written as a polynomial in t = V - V_mid,i:
-// ESDC_VTAB_NC - 1 FMAs per function.  The functions are analytic in a strip
-// about the real axis of half-width about pi k (k, sr >= 4 mV on the models'
-// parameter ranges), so the interpolation error falls like (w / (4 pi k))^NC:
-// narrow intervals allow a low degree.  Measured (FP64 Horner against long
-// double, 17 points per interval, SYN19): degree 8 on 1 mV, 7 on 1/2, 6 on
-// 1/4, 5 on 1/8 and 4 on 1/32 mV all stay at the rounding floor (at most
-// 4.0e-16 absolute for w_inf, 2.2e-16 relative for Lambda); 4 on 1/16 mV
-// reaches 2.9e-15, 3 on 1/64 mV 7.6e-15 and 3 on 1/128 mV 5.4e-16.  Fewer
-// FMAs per evaluation paid for more than the larger table (24 MB at degree 3,
-// held in L2) cost: the headline node class went from 9.53 to 9.06, 8.59,
-// 8.16, 7.28 and 6.93 ms per step along that series.  The table in use is
-// checked at 9 points per interval.
-// A table whose FP64 evaluation misses by more than ESDC_VTAB_TOL is refused
-// (the kernels then evaluate directly).  The oracle keeps the direct
-// formulas; the table is a way of computing the same functions.
+// kernel.  Here each function is replaced, on each interval of width
+// w = ESDC_VTAB_W (1/128 mV) centred at V_lo + i w, by its Chebyshev interpolant of
+// degree 3 (4 Chebyshev points, values in long double), a cubic in t = V -
+// centre that esdc_tabeval.h evaluates in FP32 pairs and integers.  The functions are
+// analytic in a strip about the real axis of half-width about pi k (k, sr >= 4 mV
+// on the models' parameter ranges), so the interpolation error falls like
+// (w / (4 pi k))^4: narrow intervals allow a low degree and leave a small bracket
+// for the FP32 pairs.  The evaluation against long double, 9 points per interval:
+// at most 5.1e-16 for w_inf (b's error over |Lambda|) and 1.5e-16 relative for
+// Lambda on SYN19, 1.5e-16 and 1.9e-16 on HH; FP64 Horner steps on the same cubics
+// made 5.4e-16, 2.3e-16, 2.2e-16 and 2.5e-16.  The table is 24 MB, held in L2.
+// A table whose evaluation misses by more than ESDC_VTAB_TOL is refused (the
+// kernels then evaluate directly).  The oracle keeps the direct formulas; the
+// table is a way of computing the same functions.
 //
-// Row i of the table (ESDC_VTAB_ROW doubles): V_mid,i, a zero pad, then for
-// each gate q the ESDC_VTAB_NC coefficient pairs (b_q, Lambda_q) of t^0, t^1,
-// ..., with b_q = -Lambda_q w_inf,q (for HH, alpha_q).  The kernels need the
+// Row i of the table (ESDC_VTAB_ROW doubles): for each gate q the cubics of b_q =
+// -Lambda_q w_inf,q (for HH, alpha_q) and of Lambda_q.  The kernels need the
 // gate's rate Lambda (u - w_inf) = Lambda u + b, one FMA from (Lambda, b);
 // w_inf itself (diagnostics) is -b / Lambda.  The error check scales b's error
 // by |Lambda|, which makes it the error in w_inf.
@@ -42,6 +36,7 @@
 #include <vector>
 
 #include "esdc_internal.h"
+#include "esdc_tabeval.h"
 
 namespace {
 
@@ -96,28 +91,17 @@ void cheb_monomial(F f, LD m, LD h, int d, LD* out)
     }
 }
 
-// Horner's rule on every second entry of c (the interleaved pairs), as the
-// kernels evaluate it.
-double horner2(const double* c, int n, double t)
-{
-    double r = c[2 * (n - 1)];
-    for (int k = n - 2; k >= 0; --k) r = std::fma(r, t, c[2 * k]);
-    return r;
-}
-
-// Rows [i0, i1) of the table; returns the largest errors of their FP64
+// Rows [i0, i1) of the table; returns the largest errors of their
 // evaluation against the direct long-double values.
 void build_rows(int model, const double* params, int i0, int i1, double* out, double& ew, double& el)
 {
-    const int NC = ESDC_VTAB_NC, d = NC - 1, NG = model == ESDC_MODEL_SYN19 ? 12 : 3;
+    const int d = 3, NG = model == ESDC_MODEL_SYN19 ? 12 : 3;
     ew = 0.0;
     el = 0.0;
-    LD coef[ESDC_VTAB_NC];
+    LD coef[4];
     for (int i = i0; i < i1; ++i) {
-        const LD lo = (LD)ESDC_VTAB_VLO + (LD)i * ESDC_VTAB_W;
-        const LD h = 0.5L * ESDC_VTAB_W, mid = lo + h;
-        double* row = out + (size_t)i * ESDC_VTAB_ROW;
-        row[0] = (double)mid;                         // exact: multiples of ESDC_VTAB_W / 2
+        const LD mid = (LD)ESDC_VTAB_VLO + (LD)i * ESDC_VTAB_W, h = 0.5L * ESDC_VTAB_W;
+        auto* row = reinterpret_cast<esdc::TabPoly*>(out + (size_t)i * ESDC_VTAB_ROW);
         for (int q = 0; q < NG; ++q) {
             const bool syn = model == ESDC_MODEL_SYN19;
             const double* p = params + (syn ? 6 * q : 0);     // SYN19: Vh, k, r, ln rho, Vr, sr
@@ -135,19 +119,20 @@ void build_rows(int model, const double* params, int i0, int i1, double* out, do
                 return -(al + be);
             };
             auto bfun = [&](LD V) { return -lam(V) * winf(V); };
-            double* cb = row + 2 + q * 2 * NC;             // b at even, Lambda at odd offsets
-            double* cl = cb + 1;
+            esdc::TabPoly &pb = row[2 * q], &pl = row[2 * q + 1];
             cheb_monomial(bfun, mid, h, d, coef);
-            for (int c = 0; c < NC; ++c) cb[2 * c] = (double)coef[c];
+            bool ok = esdc::tab_pack(coef, h, pb);
             cheb_monomial(lam, mid, h, d, coef);
-            for (int c = 0; c < NC; ++c) cl[2 * c] = (double)coef[c];
-            for (int s = 0; s <= 8; ++s) {            // the FP64 evaluation against the direct values
-                const double V = (double)(lo + (LD)ESDC_VTAB_W * s / 8.0L);
-                const double t = V - row[0];
+            ok = esdc::tab_pack(coef, h, pl) && ok;
+            if (!ok) ew = HUGE_VAL;
+            for (int s = 0; s <= 8; ++s) {            // the evaluation against the direct values
+                const double V = (double)(mid + h * (s - 4) / 4.0L);
+                float th, tl;
+                esdc::tab_split(V - (double)mid, th, tl);
                 const LD l0 = lam((LD)V), b0 = -l0 * winf((LD)V);
                 // b's error relative to |Lambda|: the error it makes in w_inf
-                ew = std::fmax(ew, (double)(fabsl((LD)horner2(cb, NC, t) - b0) / fabsl(l0)));
-                el = std::fmax(el, (double)(fabsl((LD)horner2(cl, NC, t) - l0) / fabsl(l0)));
+                ew = std::fmax(ew, (double)(fabsl((LD)esdc::tab_eval(pb, th, tl) - b0) / fabsl(l0)));
+                el = std::fmax(el, (double)(fabsl((LD)esdc::tab_eval(pl, th, tl) - l0) / fabsl(l0)));
             }
         }
     }

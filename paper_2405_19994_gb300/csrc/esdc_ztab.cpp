@@ -12,9 +12,9 @@
 // its exponent and leading mantissa bits (integer work).  The phi functions are
 // entire and their n-th derivatives fall like |z|^-(n+1) for large |z|, so the
 // interpolation error is about the same in every octave.  On each interval
-// every function is its Chebyshev interpolant of degree ESDC_ZTAB_NC - 1
-// (values in long double), stored as a polynomial in t = y - y_mid.  Beyond
-// the last octave (|z| >= 2^ESDC_ZTAB_OCT - 1) the kernels evaluate directly.
+// every function is its Chebyshev interpolant of degree 3 (values in long double),
+// a cubic in t = y - y_mid that esdc_tabeval.h evaluates in FP32 pairs and integers.
+// Beyond the last octave (|z| >= 2^ESDC_ZTAB_OCT - 1) the kernels evaluate directly.
 //
 // phi_k(x), x <= 0, in long double: for |x| <= 32 the series
 //   phi_k(x) = e^x / (k-1)! sum_m (-x)^m / (m! (m + k))
@@ -23,20 +23,16 @@
 // forward recurrence phi_{k+1} = (phi_k - 1/k!)/x, whose error shrinks by
 // k/|x| < 1 per step there.
 //
-// The table is checked when it is built: the FP64 Horner evaluation against
-// the long-double functions at 9 points per interval, the error measured in
-// units of dt (a_ij and phi_1 are of order one).  A table that misses by more
-// than ESDC_ZTAB_TOL is refused and the kernels evaluate directly.  Measured
-// (the error does not depend on dt; checked from 1e-3 to 10 ms): degree 4 on
-// 256 intervals per octave, at most 1.2e-16 for M = 4 and 2.0e-15 for M = 8;
-// degree 3 on 512 intervals per octave misses the tolerance; degree 3 on 1024
-// (12 octaves, 12288 rows, the table in use), at most 6.6e-16 for M = 4 and
-// 2.0e-15 over M = 1..8.  On the synthetic slab the set-up went from 2.90 ms
-// per step (direct) to 1.16 (degree 4) and 0.94 ms (degree 3).
+// The table is checked when it is built: its evaluation against the long-double
+// functions at 9 points per interval, the error measured in units of dt (a_ij and
+// phi_1 are of order one).  A table that misses by more than ESDC_ZTAB_TOL is refused
+// and the kernels evaluate directly.  Measured (the error does not depend on dt;
+// checked from 1e-3 to 10 ms): 12 octaves of 1024 intervals (12288 rows, the table
+// in use) at most 6.6e-16 for M = 4 and 2.0e-15 over M = 1..8, which is the cubics'
+// own interpolation error; 512 intervals per octave miss the tolerance.
 //
-// Row r of the table (ESDC_ZTAB_ROW(M) doubles): y_mid, a zero pad, then for
-// i = 0..M-1 the function dt d_{i+1} phi_1 and the M functions dt S_{i+1,j},
-// ESDC_ZTAB_NC coefficients each, lowest power first.
+// Row r of the table (ESDC_ZTAB_ROW(M) doubles): for i = 0..M-1 the cubics of
+// dt d_{i+1} phi_1 and of the M functions dt S_{i+1,j}; y_mid is the interval's.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -45,6 +41,7 @@
 #include <vector>
 
 #include "esdc_internal.h"
+#include "esdc_tabeval.h"
 
 namespace {
 
@@ -124,13 +121,6 @@ void cheb_fit(F f, int nf, LD m, LD h, int d, std::vector<LD>& out)
     }
 }
 
-double horner(const double* c, int n, double t)
-{
-    double r = c[n - 1];
-    for (int k = n - 2; k >= 0; --k) r = std::fma(r, t, c[k]);
-    return r;
-}
-
 // The M (M + 1) functions of y = 1 - z, in row order (see above).
 void functions(int M, const ColloData& C, LD dt, LD y, LD* out)
 {
@@ -151,24 +141,24 @@ void functions(int M, const ColloData& C, LD dt, LD y, LD* out)
 
 void build_rows(int M, const ColloData& C, double dt, int r0, int r1, double* rows, double& err)
 {
-    const int NC = ESDC_ZTAB_NC, nf = M * (M + 1), row_len = ESDC_ZTAB_ROW(M);
+    const int nf = M * (M + 1), row_len = ESDC_ZTAB_ROW(M);
     err = 0.0;
     std::vector<LD> coef, exact(nf);
     for (int r = r0; r < r1; ++r) {
         const int e = r >> ESDC_ZTAB_SUB, s = r & ((1 << ESDC_ZTAB_SUB) - 1);
         const LD w = ldexpl(1.0L, e - ESDC_ZTAB_SUB);     // interval width in octave e
         const LD lo = ldexpl(1.0L, e) + w * s, h = 0.5L * w, mid = lo + h;
-        double* row = rows + (size_t)r * row_len;
-        row[0] = (double)mid;                             // exact: a dyadic rational
-        cheb_fit([&](LD y, LD* v) { functions(M, C, (LD)dt, y, v); }, nf, mid, h, NC - 1, coef);
+        auto* row = reinterpret_cast<esdc::TabPoly*>(rows + (size_t)r * row_len);
+        cheb_fit([&](LD y, LD* v) { functions(M, C, (LD)dt, y, v); }, nf, mid, h, 3, coef);
         for (int q = 0; q < nf; ++q)
-            for (int p = 0; p < NC; ++p) row[2 + q * NC + p] = (double)coef[(size_t)q * NC + p];
+            if (!esdc::tab_pack(&coef[(size_t)q * 4], h, row[q])) err = HUGE_VAL;
         for (int k = 0; k <= 8; ++k) {
             const double y = (double)(lo + w * k / 8.0L);
             functions(M, C, (LD)dt, (LD)y, exact.data());
-            const double t = y - row[0];
+            float th, tl;
+            esdc::tab_split(y - (double)mid, th, tl);         // mid is exact: a dyadic rational
             for (int q = 0; q < nf; ++q) {
-                const LD got = (LD)horner(row + 2 + q * NC, NC, t);
+                const LD got = (LD)esdc::tab_eval(row[q], th, tl);
                 err = std::fmax(err, (double)(fabsl(got - exact[q]) / (LD)dt));
             }
         }
