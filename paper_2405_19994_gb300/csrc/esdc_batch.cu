@@ -468,22 +468,45 @@ __global__ void __launch_bounds__(512) k_cgb(BCgArgs a)
 // from the bound 2 q^k ||r_0|| <= tol ||b||, q = (sqrt(kappa) - 1)/(sqrt(kappa) + 1);
 // the residual is reduced (tile, then tissue, as in k_cgb) only at that
 // iteration and every second one after it, and at the cap.  One grid barrier
-// per iteration.  The same bookkeeping as k_cgb: the block holding a tissue's
+// per pass.  The same bookkeeping as k_cgb: the block holding a tissue's
 // first tile records its outcome, and the loop ends after the barrier at which
 // every tissue has recorded one.  Results per tissue depend on nothing but the
 // tissue, so batching keeps them bit for bit.  cheb_all is the solve as a
 // device function: `target` carries the grid barrier's count across the
 // phases of a persistent kernel; false means a barrier wait gave up (the
 // caller must return).
+//
+// Larger tissues iterate in FP32 (kFp32) on corrections e of (I - g L) e = r,
+// take each off the FP64 residual (kDefect: r -= B e) and add it to x in FP64,
+// to the same stop test.  An FP64 pass costs 10 FP64-pipe operations per node,
+// 85 us for the 64 tissues of 64 to 512 nodes a side (5.1M nodes) where its
+// bytes take 40; an FP32 pass moves half the bytes and leaves that pipe alone.
+// 64 tissues of 64..512 nodes a side 32.3 -> 28.3 ms per step, 16 slices of 256x256 10.5 -> 9.0 ms per
+// Q^par solve.
+// A correction reduces the residual by 3e-6 at most (kFmin2; FP32's rounding
+// leaves about kappa 6e-8, kappa at most 64), so a warm-started solve takes one
+// or two.  The last one's FP32 residual tells whether it met the test, with
+// 2e-6 ||r|| as the allowance for its rounding; else the FP64 residual decides.
+// What FP32 cannot do (a residual out of its range, no progress) the FP64
+// iterations finish (kStart64, kFp64).  The defect pass and its barrier are
+// what it costs, so small tissues, which the barriers bound, stay in FP64; the
+// line depends on the tissue alone, as its results do.
+enum : int { kStop = 0, kFp64, kFp32, kDefect, kStart64 };
+constexpr int kRefMinNodes = 16385;      // nodes of a tissue from which it iterates in FP32
+constexpr int kRefMaxOut = 8;            // corrections before the FP64 iterations take over
+constexpr double kFmin2 = 1e-11;         // least reduction (squared) asked of one correction
+
 __device__ bool cheb_all(const BCgArgs& a, unsigned& target)
 {
     constexpr int U = ESDC_TILE / 32;
-    __shared__ bool s_active[kMaxBlockTissues], s_chk[kMaxBlockTissues];
+    __shared__ bool s_chk[kMaxBlockTissues], s_ref[kMaxBlockTissues], s_final[kMaxBlockTissues];
+    __shared__ int s_mode[kMaxBlockTissues], s_it[kMaxBlockTissues], s_chunk[kMaxBlockTissues];
+    __shared__ int s_first[kMaxBlockTissues], s_out[kMaxBlockTissues];
+    __shared__ unsigned s_magx[kMaxBlockTissues], s_magy[kMaxBlockTissues];
     __shared__ double s_gih2[kMaxBlockTissues], s_diag[kMaxBlockTissues][8];
     __shared__ double s_s1[kMaxBlockTissues], s_delta[kMaxBlockTissues], s_rho[kMaxBlockTissues];
     __shared__ double s_ca[kMaxBlockTissues], s_cb[kMaxBlockTissues], s_stop[kMaxBlockTissues];
-    __shared__ double s_itheta[kMaxBlockTissues];
-    __shared__ int s_chunk[kMaxBlockTissues];
+    __shared__ double s_itheta[kMaxBlockTissues], s_rr[kMaxBlockTissues], s_logq[kMaxBlockTissues];
     __shared__ double s_tot[kMaxBlockTissues * 2];
     __shared__ int s_exit;
 
@@ -515,29 +538,46 @@ __device__ bool cheb_all(const BCgArgs& a, unsigned& target)
         s_delta[k] = delta;
         s_itheta[k] = 1.0 / theta;
         s_s1[k] = delta > 0.0 ? theta / delta : 0.0;
-        s_rho[k] = delta > 0.0 ? delta / theta : 0.0;        // rho_0
-        s_active[k] = true;
+        // kappa = 1 + 2 delta at most 64
+        s_ref[k] = T->N >= kRefMinNodes && delta > 0.0 && delta <= 31.5 && a.tol2 > 0.0;
+        s_mode[k] = kFp64;
+        s_chk[k] = true;
+        s_it[k] = 0;
+        s_out[k] = 0;
+        // q / n = umulhi(q, floor(2^32/n)) or one more (0 <= q < 2^31; n = 1: 2^32 - 1)
+        s_magx[k] = T->nx > 1 ? (unsigned)(0x100000000ull / (unsigned)T->nx) : 0xffffffffu;
+        s_magy[k] = T->ny > 1 ? (unsigned)(0x100000000ull / (unsigned)T->ny) : 0xffffffffu;
         if (T->tile0 >= bt.t0 && T->tile0 < bt.t1) a.done_at[bt.lo + k] = INT_MAX;
     }
     __syncthreads();
 
-    auto op = [&](const double* v, int p, const TileGeo& G, int k) -> double {
-        const int q = p - G.off;
-        const int r = q / G.nx;
-        const int ix = q - r * G.nx;
-        const int iz = r / G.ny;
-        const int iy = r - iz * G.ny;
+    // The sum of node q's neighbours in its tissue's array v (as TO) and their number.
+    auto neighbours = [&](auto get, int q, const TileGeo& G, int k, auto& s) -> int {
+        int r = (int)__umulhi((unsigned)q, s_magx[k]), ix = q - r * G.nx;
+        if (ix >= G.nx) { ix -= G.nx; ++r; }
+        int iz = (int)__umulhi((unsigned)r, s_magy[k]), iy = r - iz * G.ny;
+        if (iy >= G.ny) { iy -= G.ny; ++iz; }
         const int sxy = G.nx * G.ny;
-        const double vp = __ldcg(v + p);
-        double s = 0.0;
         int c = 0;
-        if (ix > 0)        { s += __ldcg(v + p - 1); ++c; }
-        if (ix < G.nx - 1) { s += __ldcg(v + p + 1); ++c; }
-        if (iy > 0)        { s += __ldcg(v + p - G.nx); ++c; }
-        if (iy < G.ny - 1) { s += __ldcg(v + p + G.nx); ++c; }
-        if (iz > 0)        { s += __ldcg(v + p - sxy); ++c; }
-        if (iz < G.nz - 1) { s += __ldcg(v + p + sxy); ++c; }
+        s = 0;
+        if (ix > 0)        { s += get(q - 1); ++c; }
+        if (ix < G.nx - 1) { s += get(q + 1); ++c; }
+        if (iy > 0)        { s += get(q - G.nx); ++c; }
+        if (iy < G.ny - 1) { s += get(q + G.nx); ++c; }
+        if (iz > 0)        { s += get(q - sxy); ++c; }
+        if (iz < G.nz - 1) { s += get(q + sxy); ++c; }
+        return c;
+    };
+    // (I - g L) v at node q: v in FP64 (its value there is vp), or in FP32 widened
+    auto op = [&](const double* v, double vp, int q, const TileGeo& G, int k) -> double {
+        double s;
+        const int c = neighbours([&](int j) { return __ldcg(v + j); }, q, G, k, s);
         return fma(s_diag[k][c], vp, -(s_gih2[k] * s));
+    };
+    auto op_wide = [&](const float* v, int q, const TileGeo& G, int k) -> double {
+        double s;
+        const int c = neighbours([&](int j) { return widen(__ldcg(v + j)); }, q, G, k, s);
+        return fma(s_diag[k][c], widen(__ldcg(v + q)), -(s_gih2[k] * s));
     };
     auto tile_geo = [&](long long t, int& k) -> TileGeo {
         const int b = a.tile_tissue[t];
@@ -548,24 +588,77 @@ __device__ bool cheb_all(const BCgArgs& a, unsigned& target)
         G.nx = T->nx; G.ny = T->ny; G.nz = T->nz; G.N = T->N; G.off = T->off;
         return G;
     };
-    double* dc = a.p;                 // d_k
-    double* dn = a.q;                 // d_{k+1}
+    // A tissue in FP32 keeps its four FP32 vectors in its own part of the FP64 vectors that it does
+    // not use: d_k and d_{k+1} in p's, e and the FP32 residual in z's (a multiple of 512 nodes each).
+    auto pad = [&](const TileGeo& G) { return (G.N + ESDC_TILE - 1) & ~(ESDC_TILE - 1); };
+    bool odd = false;                 // d_k is in a.q (FP32: the second half), d_{k+1} in a.p (the first)
+
+    // Decisions on tissue k, by one thread, the same in every block that holds a part of it.
+    int tick = -1;                    // passes of the loop below
+    auto stop_tissue = [&](int k, int f) {
+        s_mode[k] = kStop;
+        const TissueDev* T = a.tis + bt.lo + k;
+        if (T->tile0 >= bt.t0 && T->tile0 < bt.t1) {
+            a.done_at[bt.lo + k] = tick;
+            a.status[2 * (bt.lo + k)] = s_it[k];
+            a.status[2 * (bt.lo + k) + 1] = f;
+            if (a.iter_log) a.iter_log[bt.lo + k] = s_it[k];
+            if (f) atomicOr(a.flags, f);
+        }
+    };
+    // Iterations that reduce the residual by f (2 q^k <= f), at least one and at most those left to the cap.
+    auto iterations = [&](int k, double f) -> int {
+        const int left = a.maxit - s_it[k];
+        if (!(s_logq[k] < 0.0)) return 1;
+        const double kd = f > 0.0 ? ceil(log(0.5 * f) / s_logq[k]) : (double)left;
+        const int kn = kd < (double)left ? (int)kd : left;
+        return kn < 1 ? 1 : kn;
+    };
+    auto start64 = [&](int k) {
+        s_mode[k] = kFp64;
+        s_chunk[k] = s_it[k] + iterations(k, sqrt(s_stop[k] / s_rr[k]));
+        s_rho[k] = s_delta[k] > 0.0 ? s_delta[k] / (1.0 + s_delta[k]) : 0.0;      // rho_0
+    };
+    // This correction's share of the reduction to a tenth of the stop test (what FP64 iterations
+    // to the bound reach): all of it if one correction can, else the square root of what is left.
+    auto start32 = [&](int k) {
+        const double f2 = 0.01 * s_stop[k] / s_rr[k];
+        s_final[k] = f2 >= kFmin2;
+        s_mode[k] = kFp32;
+        s_first[k] = s_it[k];
+        s_chunk[k] = s_it[k] + iterations(k, sqrt(s_final[k] ? f2 : fmax(sqrt(f2), kFmin2)));
+        s_rho[k] = s_delta[k] / (1.0 + s_delta[k]);
+    };
+    // FP32's range: the squares of a residual of rms 1e-13 to 1e13, reduced by 3e-6, stay in it
+    auto in_range = [&](int k, double rr) {
+        const double n = a.tis[bt.lo + k].N;
+        return rr > 1e-26 * n && rr < 1e26 * n;
+    };
 
     // [S] r = b - B x, d_0 = r / theta; tile partials r.r, b.b (slots 0-1)
     for (long long t = wt0; t < wt1; ++t) {
         int k;
         const TileGeo G = tile_geo(t, k);
         const double inv_theta = s_itheta[k];
+        const bool ref = s_ref[k];
+        float* df = reinterpret_cast<float*>(a.p + G.off);
+        float* zf = reinterpret_cast<float*>(a.z + G.off) + pad(G);
         double v0 = 0.0, v1 = 0.0;
 #pragma unroll 4
         for (int u = 0; u < U; ++u) {
-            const int p = G.base + lane + 32 * u;
-            if (p - G.off >= G.N) continue;
-            const double bx = op(a.x, p, G, k);
+            const int p = G.base + lane + 32 * u, q = p - G.off;
+            if (q >= G.N) continue;
+            const double bx = op(a.x + G.off, __ldcg(a.x + p), q, G, k);
             const double bp = __ldcg(a.b + p);
             const double rp = bp - bx;
             a.r[p] = rp;
-            dc[p] = rp * inv_theta;
+            if (ref) {
+                const float rf = (float)rp;
+                zf[q] = rf;
+                df[q] = rf * (float)inv_theta;
+            } else {
+                a.p[p] = rp * inv_theta;
+            }
             v0 = fma(rp, rp, v0);
             v1 = fma(bp, bp, v1);
         }
@@ -576,112 +669,154 @@ __device__ bool cheb_all(const BCgArgs& a, unsigned& target)
         }
     }
     if (!grid_barrier(a.bar, target, a.flags)) return false;
-    tissue_totals(a, bt, s_active, 0, 2, s_tot);
-    if (threadIdx.x == 0) {
-        for (int k = 0; k < bt.n; ++k) {
-            const double rr = s_tot[2 * k], stop = a.tol2 * s_tot[2 * k + 1];
-            s_stop[k] = stop;
-            const bool bad = !isfinite(rr) || !isfinite(stop);
-            const bool conv = rr <= stop;
-            if (bad || conv) {
-                s_active[k] = false;
-                const TissueDev* T = a.tis + bt.lo + k;
-                if (T->tile0 >= bt.t0 && T->tile0 < bt.t1) {
-                    a.done_at[bt.lo + k] = -1;
-                    a.status[2 * (bt.lo + k)] = 0;
-                    a.status[2 * (bt.lo + k) + 1] = bad ? ESDC_FLAG_NONFINITE : 0;
-                    if (a.iter_log) a.iter_log[bt.lo + k] = 0;
-                    if (bad) atomicOr(a.flags, ESDC_FLAG_NONFINITE);
-                }
-                continue;
-            }
-            // iterations the bound asks for (tol 0: up to the cap)
-            int kn = 1;
-            const double kap = 1.0 + 2.0 * s_delta[k];
-            const double q = (sqrt(kap) - 1.0) / (sqrt(kap) + 1.0);
-            if (q > 0.0) {
-                const double kd = stop > 0.0 ? ceil(log(0.5 * sqrt(stop / rr)) / log(q)) : (double)a.maxit;
-                kn = kd < (double)a.maxit ? (int)kd : a.maxit;
-            }
-            s_chunk[k] = kn < 1 ? 1 : kn;
-        }
+    tissue_totals(a, bt, s_chk, 0, 2, s_tot);
+    for (int k = threadIdx.x; k < bt.n; k += blockDim.x) {
+        const double rr = s_tot[2 * k], stop = a.tol2 * s_tot[2 * k + 1];
+        s_stop[k] = stop;
+        s_rr[k] = rr;
+        const double kap = 1.0 + 2.0 * s_delta[k];
+        s_logq[k] = kap > 1.0 ? log((sqrt(kap) - 1.0) / (sqrt(kap) + 1.0)) : 0.0;
+        if (!isfinite(rr) || !isfinite(stop)) stop_tissue(k, ESDC_FLAG_NONFINITE);
+        else if (rr <= stop) stop_tissue(k, 0);
+        else if (!s_ref[k]) start64(k);                       // d_0 is there
+        else if (stop > 0.0 && in_range(k, rr)) start32(k);
+        else s_mode[k] = kStart64;
     }
     __syncthreads();
 
-    for (int it = 0;; ++it) {
-        if (it > a.maxit) {                   // cannot happen: every tissue stops by maxit
+    for (tick = 0;; ++tick) {
+        if (tick > a.maxit + kRefMaxOut + 1) {                // cannot happen: every tissue stops by maxit
             if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(a.flags, ESDC_FLAG_CG_MAXIT);
             break;
         }
         // this iteration's coefficients, and which tissues check their residual after it
         for (int k = threadIdx.x; k < bt.n; k += blockDim.x) {
-            if (!s_active[k]) { s_chk[k] = false; continue; }
+            const int mode = s_mode[k];
+            s_chk[k] = mode == kDefect;
+            if (mode != kFp64 && mode != kFp32) continue;
             const double rho = s_rho[k];
             const double rn = s_delta[k] > 0.0 ? 1.0 / (2.0 * s_s1[k] - rho) : 0.0;
             s_ca[k] = rn * rho;
             s_cb[k] = s_delta[k] > 0.0 ? 2.0 * rn / s_delta[k] : 0.0;
             s_rho[k] = rn;
-            s_chk[k] = it + 1 >= s_chunk[k] || it + 1 >= a.maxit;
+            s_chk[k] = s_it[k] + 1 >= s_chunk[k] || s_it[k] + 1 >= a.maxit;
         }
         __syncthreads();
-        // [U] x += d, r -= B d, d' = ca d + cb r; tile partials r.r of the checking tissues (slot 2)
+        // [U] the tissue's pass; tile partials r.r of the checking tissues (slot 2)
+        double* dc = odd ? a.q : a.p;
+        double* dn = odd ? a.p : a.q;
         for (long long t = wt0; t < wt1; ++t) {
             int k;
             const TileGeo G = tile_geo(t, k);
-            if (!s_active[k]) continue;
-            const double ca = s_ca[k], cb = s_cb[k];
+            const int mode = s_mode[k];
+            if (mode == kStop) continue;
             const bool chk = s_chk[k];
+            const int q0 = G.base - G.off + lane;
             double v = 0.0;
+            if (mode == kFp64) {
+                // x += d, r -= B d, d' = ca d + cb r
+                const double ca = s_ca[k], cb = s_cb[k];
 #pragma unroll 4
-            for (int u = 0; u < U; ++u) {
-                const int p = G.base + lane + 32 * u;
-                if (p - G.off >= G.N) continue;
-                const double bd = op(dc, p, G, k);
-                const double dp = __ldcg(dc + p);
-                const double rp = __ldcg(a.r + p) - bd;
-                a.x[p] = __ldcg(a.x + p) + dp;
-                a.r[p] = rp;
-                dn[p] = fma(ca, dp, cb * rp);
-                if (chk) v = fma(rp, rp, v);
+                for (int u = 0; u < U; ++u) {
+                    const int q = q0 + 32 * u, p = G.off + q;
+                    if (q >= G.N) continue;
+                    const double dp = __ldcg(dc + p);
+                    const double bd = op(dc + G.off, dp, q, G, k);
+                    const double rp = __ldcg(a.r + p) - bd;
+                    a.x[p] = __ldcg(a.x + p) + dp;
+                    a.r[p] = rp;
+                    dn[p] = fma(ca, dp, cb * rp);
+                    if (chk) v = fma(rp, rp, v);
+                }
+            } else if (mode == kStart64) {
+                const double inv_theta = s_itheta[k];
+                for (int q = q0; q < q0 + ESDC_TILE && q < G.N; q += 32) dn[G.off + q] = __ldcg(a.r + G.off + q) * inv_theta;
+            } else {
+                float* df = reinterpret_cast<float*>(a.p + G.off);
+                float* ef = reinterpret_cast<float*>(a.z + G.off);
+                float* zf = ef + pad(G);
+                float* dcf = odd ? df + pad(G) : df;
+                float* dnf = odd ? df : df + pad(G);
+                if (mode == kFp32) {
+                    // e += d, r -= B d, d' = ca d + cb r; the last one adds e to x
+                    const float ca = (float)s_ca[k], cb = (float)s_cb[k], gf = (float)s_gih2[k];
+                    const bool first = s_it[k] == s_first[k];
+                    float acc = 0.0f;
+#pragma unroll 4
+                    for (int u = 0; u < U; ++u) {
+                        const int q = q0 + 32 * u;
+                        if (q >= G.N) continue;
+                        float s;
+                        const int c = neighbours([&](int j) { return dcf[j]; }, q, G, k, s);
+                        const float d = dcf[q];
+                        const float rn = zf[q] - fmaf(fmaf(gf, (float)c, 1.0f), d, -(gf * s));
+                        const float en = first ? d : ef[q] + d;
+                        ef[q] = en;
+                        if (chk) {
+                            const double xp = a.x[G.off + q];
+                            a.x[G.off + q] = xp + widen(en);
+                            acc = fmaf(rn, rn, acc);
+                        } else {
+                            zf[q] = rn;
+                            dnf[q] = fmaf(ca, d, cb * rn);
+                        }
+                    }
+                    v = acc;
+                } else {
+                    // kDefect: r -= B e in FP64, and the next correction's start
+                    const float inv_theta = (float)s_itheta[k];
+#pragma unroll 4
+                    for (int u = 0; u < U; ++u) {
+                        const int q = q0 + 32 * u, p = G.off + q;
+                        if (q >= G.N) continue;
+                        const double rp = __ldcg(a.r + p) - op_wide(ef, q, G, k);
+                        a.r[p] = rp;
+                        const float rf = (float)rp;
+                        zf[q] = rf;
+                        dnf[q] = rf * inv_theta;
+                        v = fma(rp, rp, v);
+                    }
+                }
             }
             if (chk) {
                 v = warp_tree(v);
                 if (lane == 0) a.part[2 * (size_t)a.ntiles + t] = v;
             }
         }
-        double* sw = dc; dc = dn; dn = sw;
+        odd = !odd;
         if (!grid_barrier(a.bar, target, a.flags)) return false;
         // every tissue has stopped by the previous iteration: leave (the same decision in every block)
         if (threadIdx.x < 32) {
             bool all = true;
-            for (int b = threadIdx.x; b < a.ntis; b += 32) all &= __ldcg(a.done_at + b) <= it - 1;
+            for (int b = threadIdx.x; b < a.ntis; b += 32) all &= __ldcg(a.done_at + b) <= tick - 1;
             all = __all_sync(0xffffffffu, all);
             if (threadIdx.x == 0) s_exit = all;
         }
         __syncthreads();
         if (s_exit) break;
         tissue_totals(a, bt, s_chk, 2, 1, s_tot);
-        if (threadIdx.x == 0) {
-            for (int k = 0; k < bt.n; ++k) {
-                if (!s_chk[k]) continue;
-                const double rr = s_tot[k];
-                const bool bad = !isfinite(rr);
-                const bool conv = rr <= s_stop[k];
-                const bool maxed = it + 1 >= a.maxit;
-                if (bad || conv || maxed) {
-                    s_active[k] = false;
-                    const TissueDev* T = a.tis + bt.lo + k;
-                    if (T->tile0 >= bt.t0 && T->tile0 < bt.t1) {
-                        const int f = bad ? ESDC_FLAG_NONFINITE : (conv ? 0 : ESDC_FLAG_CG_MAXIT);
-                        a.done_at[bt.lo + k] = it;
-                        a.status[2 * (bt.lo + k)] = it + 1;
-                        a.status[2 * (bt.lo + k) + 1] = f;
-                        if (a.iter_log) a.iter_log[bt.lo + k] = it + 1;
-                        if (f) atomicOr(a.flags, f);
-                    }
-                } else {
-                    s_chunk[k] = it + 3;          // rounding left it short: two more, then check
-                }
+        for (int k = threadIdx.x; k < bt.n; k += blockDim.x) {
+            const int mode = s_mode[k];
+            if (mode == kStart64) { start64(k); continue; }
+            if (mode == kFp64 || mode == kFp32) ++s_it[k];
+            if (!s_chk[k]) continue;
+            const double rr = s_tot[k];
+            if (!isfinite(rr)) {
+                stop_tissue(k, ESDC_FLAG_NONFINITE);
+            } else if (mode == kFp32) {
+                if (s_final[k] && sqrt(rr) + 2e-6 * sqrt(s_rr[k]) <= sqrt(s_stop[k])) stop_tissue(k, 0);
+                else s_mode[k] = kDefect;
+            } else if (rr <= s_stop[k]) {
+                stop_tissue(k, 0);
+            } else if (s_it[k] >= a.maxit) {
+                stop_tissue(k, ESDC_FLAG_CG_MAXIT);
+            } else if (mode == kFp64) {
+                s_chunk[k] = s_it[k] + 2;             // rounding left it short: two more, then check
+            } else {
+                const bool on = rr <= 1e-2 * s_rr[k] && in_range(k, rr) && ++s_out[k] < kRefMaxOut;
+                s_rr[k] = rr;
+                if (on) start32(k);
+                else s_mode[k] = kStart64;            // no progress: FP64 from here
             }
         }
         __syncthreads();
@@ -689,7 +824,12 @@ __device__ bool cheb_all(const BCgArgs& a, unsigned& target)
     return true;
 }
 
-__global__ void __launch_bounds__(512, 1) k_chebb(BCgArgs a)
+// PER_SM: blocks of 512 threads that the registers allow per SM.  One (104 registers, more loads
+// in flight per warp) while a 512-thread block per SM has a warp for every tile, else two (64):
+// 16 slices of 256x256 (2048 tiles) 9.12 / 9.28 ms per Q^par solve, 64 tissues of 64..512 nodes a
+// side (9,900 tiles) 31.4 / 28.5 ms per step.
+template <int PER_SM>
+__global__ void __launch_bounds__(512, PER_SM) k_chebb(BCgArgs a)
 {
     unsigned target = 0;
     cheb_all(a, target);
@@ -829,6 +969,7 @@ struct esdc_batch {
     unsigned long long* rmax = nullptr;    // [ntis][2 NS]
     // launch shapes (esdc_batch_tune)
     int node_waves = 1, cg_threads = 512, cg_blocks = 0;
+    int cg_launch = 512;                   // threads per solve block: cg_threads, or auto_threads
     int occ_node[ESDC_MMAX + 1] = {0}, occ_setup[ESDC_MMAX + 1] = {0}, occ_res[ESDC_MMAX + 1] = {0},
         occ_iter[ESDC_MMAX + 1] = {0};
     // one persistent launch per step (k_bstep; Chebyshev solves only): on/off,
@@ -903,9 +1044,13 @@ int max_block_tissues(const esdc_batch* b, int nb, int threads)
     return worst;
 }
 
+// Whether the tiles are more than one 512-thread block per SM has warps.
+bool many_tiles(const esdc_batch* b) { return b->ntiles > b->sms * 16; }
+
 int cg_grid(const esdc_batch* b, int threads, int per_sm_wanted)
 {
-    const int occ = b->opt.solver == 0 ? occupancy(k_chebb, threads) : occupancy(k_cgb, threads);
+    const int occ = b->opt.solver != 0 ? occupancy(k_cgb, threads)
+                  : many_tiles(b) ? occupancy(k_chebb<2>, threads) : occupancy(k_chebb<1>, threads);
     if (occ < 1) return 0;
     int per_sm = std::min(occ, per_sm_wanted);
     long long nb = (long long)b->sms * per_sm;
@@ -913,6 +1058,18 @@ int cg_grid(const esdc_batch* b, int threads, int per_sm_wanted)
     nb = std::max(1LL, std::min(nb, need));
     while (nb > 1 && max_block_tissues(b, (int)nb, threads) > kMaxBlockTissues) --nb;
     return (int)nb;
+}
+
+// The solve's shape until esdc_batch_set_shape gives one: a warp takes whole tiles, so the blocks
+// have as many warps as it takes to give every SM its share of the tiles, 16 at most (then two
+// blocks per SM).  With 512-thread blocks throughout, the 32 tiles of a 128x128 sheet ran on two of
+// the 152 SMs.
+void auto_shape(esdc_batch* b)
+{
+    const int warps = std::max(1, std::min(16, (b->ntiles + b->sms - 1) / b->sms));
+    b->cg_threads = 512;
+    b->cg_launch = 32 * warps;
+    b->cg_blocks = cg_grid(b, b->cg_launch, b->opt.solver == 0 && many_tiles(b) ? 2 : 1);
 }
 
 // The step's kernel arguments for M collocation nodes and step dt (the
@@ -992,8 +1149,8 @@ cudaError_t launch_cgb(esdc_batch* b, double gfac, const double* rhs, double* x,
     void* args[] = {&a};
     cudaError_t e = cudaMemsetAsync(b->bar, 0, sizeof(unsigned), s);
     if (e != cudaSuccess) return e;
-    const void* k = b->opt.solver == 0 ? (const void*)k_chebb : (const void*)k_cgb;
-    return cudaLaunchCooperativeKernel(k, dim3(b->cg_blocks), dim3(b->cg_threads), args, 0, s);
+    const void* k = b->opt.solver != 0 ? (const void*)k_cgb : many_tiles(b) ? (const void*)k_chebb<2> : (const void*)k_chebb<1>;
+    return cudaLaunchCooperativeKernel(k, dim3(b->cg_blocks), dim3(b->cg_launch), args, 0, s);
 }
 
 // Occupancy of the step kernels (queried before any stream capture).
@@ -1372,10 +1529,9 @@ int esdc_batch_create(int n, const esdc_mesh* meshes, const double* sigma, doubl
     cudaMemset(b->status, 0, sizeof(int) * 2 * n);
     cudaMemset(b->cg_log, 0, sizeof(int) * b->cg_log_len);
     cudaMemset(b->flags, 0, sizeof(int));
-    b->cg_threads = 512;
-    b->cg_blocks = cg_grid(b, b->cg_threads, 1);
+    auto_shape(b);
     if (b->cg_blocks < 1) return fail(ESDC_ERR_CUDA);
-    if (max_block_tissues(b, b->cg_blocks, b->cg_threads) > kMaxBlockTissues) return fail(ESDC_ERR_UNSUPPORTED);
+    if (max_block_tissues(b, b->cg_blocks, b->cg_launch) > kMaxBlockTissues) return fail(ESDC_ERR_UNSUPPORTED);
     if (cudaDeviceSynchronize() != cudaSuccess) return fail(ESDC_ERR_CUDA);
     *out = b;
     return ESDC_OK;
@@ -1611,7 +1767,7 @@ int esdc_batch_set_shape(esdc_batch* b, int node_waves, int cg_threads, int cg_b
     cudaDeviceSynchronize();
     drop_graph(b);
     b->node_waves = node_waves;
-    b->cg_threads = cg_threads;
+    b->cg_threads = b->cg_launch = cg_threads;
     b->cg_blocks = nb;
     return ESDC_OK;
 }
@@ -1626,9 +1782,10 @@ int esdc_batch_tune(esdc_batch* b, double* y_scratch, double V0, double t, doubl
     // Candidates: the launch sequence with its launch shapes (node-kernel waves,
     // solve block size and blocks per SM), and, with the Chebyshev solves, the
     // persistent step kernel with its block size and node tile.  None changes
-    // a bit of the results.
+    // a bit of the results.  threads 0: the automatic solve shape.
     struct Shape { int persist, waves, threads, per_sm, tile; };
-    const Shape cand[] = {{0, 1, 512, 1, 0}, {0, 2, 512, 1, 0}, {0, 4, 512, 1, 0}, {0, 1, 256, 1, 0},
+    const Shape cand[] = {{0, 1, 0, 0, 0}, {0, 4, 0, 0, 0}, {0, 1, 512, 1, 0}, {0, 2, 512, 1, 0}, {0, 4, 512, 1, 0}, {0, 1, 512, 2, 0},
+                          {0, 2, 512, 2, 0}, {0, 4, 512, 2, 0}, {0, 1, 256, 1, 0},
                           {0, 1, 256, 2, 0}, {0, 2, 256, 2, 0}, {0, 4, 256, 2, 0},
                           {1, 0, 512, 0, 32}, {1, 0, 512, 0, 128}, {1, 0, 512, 0, 512},
                           {1, 0, 256, 0, 32}, {1, 0, 256, 0, 64}, {1, 0, 256, 0, 128}};
@@ -1649,7 +1806,10 @@ int esdc_batch_tune(esdc_batch* b, double* y_scratch, double V0, double t, doubl
             if (esdc_batch_set_persistent(b, 1, c.threads, c.tile) != ESDC_OK) continue;
         } else {
             if (esdc_batch_set_persistent(b, 0, b->p_threads, b->p_tile) != ESDC_OK) continue;
-            if (esdc_batch_set_shape(b, c.waves, c.threads, c.per_sm) != ESDC_OK) continue;
+            if (c.threads == 0) {
+                b->node_waves = c.waves;
+                auto_shape(b);
+            } else if (esdc_batch_set_shape(b, c.waves, c.threads, c.per_sm) != ESDC_OK) continue;
         }
         rc = esdc_batch_init_state(b, y_scratch, V0, stream);
         if (rc == ESDC_OK) rc = esdc_batch_sweep(b, y_scratch, tv.data(), dt, M, K, stream);   // capture, warm-up
@@ -1679,8 +1839,11 @@ int esdc_batch_tune(esdc_batch* b, double* y_scratch, double V0, double t, doubl
     } else {
         b->persist = 0;
         b->node_waves = pick.waves ? pick.waves : seq0.waves;
-        b->cg_threads = pick.threads;
-        b->cg_blocks = pick_blocks;
+        auto_shape(b);
+        if (pick.threads) {
+            b->cg_threads = b->cg_launch = pick.threads;
+            b->cg_blocks = pick_blocks;
+        }
     }
     return ESDC_OK;
 }

@@ -45,16 +45,6 @@ __device__ __forceinline__ Q4<float> ld4(const float* a)
     return {{u.x, u.y, u.z, u.w}};
 }
 
-// FP32 value as FP64 by integer operations (the FP64 pipe also does the
-// conversions, at its own rate): exact for normal numbers and zero, FP32
-// subnormals become zero; not for Inf and NaN.
-__device__ __forceinline__ double widen(float f)
-{
-    const unsigned u = __float_as_uint(f), a = u & 0x7fffffffu;
-    const bool z = a < 0x00800000u;
-    return __hiloint2double((int)((u & 0x80000000u) | (z ? 0u : (a >> 3) + 0x38000000u)), z ? 0 : (int)(u << 29));
-}
-
 // A value, and a quad, of storage type S as type T.
 template <typename T, typename S> struct Load {
     static __device__ __forceinline__ T one(const S* a) { return __ldcg(a); }

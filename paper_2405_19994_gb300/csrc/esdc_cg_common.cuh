@@ -172,6 +172,16 @@ __device__ void grid_total_q(const double* part, int off0, double (&tot)[NV], do
     __syncthreads();
 }
 
+// FP32 value as FP64 by integer operations (the FP64 pipe also does the
+// conversions, at its own rate): exact for normal numbers and zero, FP32
+// subnormals become zero; not for Inf and NaN.
+__device__ __forceinline__ double widen(float f)
+{
+    const unsigned u = __float_as_uint(f), a = u & 0x7fffffffu;
+    const bool z = a < 0x00800000u;
+    return __hiloint2double((int)((u & 0x80000000u) | (z ? 0u : (a >> 3) + 0x38000000u)), z ? 0 : (int)(u << 29));
+}
+
 struct NodeIdx { int ix, iy, iz; };
 
 __device__ __forceinline__ NodeIdx node_idx(const MeshDev& m, int p)
