@@ -32,7 +32,11 @@
 //    It is solved directly (Thomas' elimination) with its factors tabulated
 //    once per value of g: r'_k = r_k A_k - r'_{k-1} C_k, x_k = r'_k - C_k x_{k+1},
 //    three FP64 operations per node.  A 2D or 1D mesh has nz = 1, where this
-//    reduces to the division by a.  When the y-z slab of one x-mode fits a
+//    reduces to the division by a.
+//  * The last transformed axis goes forward, through the division and back in one
+//    kernel (k_dct_last) where it is an FFT axis and nothing lies between: 1D and
+//    2D meshes, and the fourth-order stencil.
+//  * When the y-z slab of one x-mode fits a
 //    block (ny a power of two >= 16, nz >= 2), k_dct_yzy does the y forward
 //    transform, these z solves and the y inverse transform of that x-mode in
 //    shared memory: three kernels per solve (x forward, yzy, x inverse).
@@ -194,6 +198,55 @@ __device__ __forceinline__ double2* fft_pow2(double2* x, double2* y, int n, int 
 // Position of x[i] in Makhoul's reordering v[m] = x[2m], v[n-1-m] = x[2m+1].
 __device__ __forceinline__ int makhoul_pos(int i, int n) { return (i & 1) ? n - 1 - (i >> 1) : (i >> 1); }
 
+// The real rows X[0..n-1] of a pair's two lines from its transform z, by the pair's G threads:
+// X[k] = Re(e^{-i th_k} V[k]), th_k = pi k/(2n); P = Z[k] + conj(Z[n-k]) = 2 Va[k],
+// Q = Z[k] - conj(Z[n-k]) = 2i Vb[k]; csh holds (cos, sin)/2.
+__device__ __forceinline__ void dct_post(const double2* z, double* ra, double* rb, int n, int g, int G,
+                                         const double2* csh)
+{
+    const int h = n >> 1;
+    for (int k = g; k <= h; k += G) {
+        if (k == 0) { ra[0] = z[0].x; rb[0] = z[0].y; continue; }
+        const double2 Zk = z[k], Zm = z[n - k];
+        const double Pr = Zk.x + Zm.x, Pi = Zk.y - Zm.y;
+        const double Qr = Zk.x - Zm.x, Qi = Zk.y + Zm.y;
+        const double2 t = __ldg(csh + k);
+        ra[k] = fma(t.x, Pr, t.y * Pi);
+        rb[k] = fma(t.x, Qi, -t.y * Qr);
+        if (k < h) {
+            ra[n - k] = fma(t.y, Pr, -t.x * Pi);
+            rb[n - k] = fma(t.y, Qi, t.x * Qr);
+        }
+    }
+}
+
+// The inverse's packing: Z[k] = conj(Va[k] + i Vb[k]), Va[k] = e^{i th_k}(A[k] - i A[n-k])
+// (A[n] = 0), and Z[n-k] from Va[n-k] = conj(Va[k]), for the real rows A (ra) and B (rb).
+__device__ __forceinline__ void dct_pack(const double* ra, const double* rb, double2* x, int n, int g, int G,
+                                         const double2* cs)
+{
+    const int h = n >> 1;
+    for (int k = g; k <= h; k += G) {
+        if (k == 0) { x[0] = make_double2(ra[0], -rb[0]); continue; }
+        const double Akx = ra[k], Aky = rb[k], Amx = ra[n - k], Amy = rb[n - k];
+        const double2 t = __ldg(cs + k);
+        const double ar = fma(t.x, Akx, t.y * Amx), ai = fma(t.y, Akx, -t.x * Amx);
+        const double br = fma(t.x, Aky, t.y * Amy), bi = fma(t.y, Aky, -t.x * Amy);
+        x[k] = make_double2(ar - bi, -(ai + br));
+        if (k < h) x[n - k] = make_double2(ar + bi, ai - br);
+    }
+}
+
+// The real rows of the inverse: conj(FFT(conj Z)), undone from the reordering.
+__device__ __forceinline__ void dct_unpack(const double2* z, double* ra, double* rb, int n, int g, int G)
+{
+    for (int i = g; i < n; i += G) {
+        const double2 v = z[makhoul_pos(i, n)];
+        ra[i] = v.x;
+        rb[i] = -v.y;
+    }
+}
+
 // One tile of lines along one axis, FFT path.  FWD: X = U x (unnormalised
 // DCT-II).  !FWD: y = U^T diag(1, 1/2, ..., 1/2) Y.  Shared memory: two
 // complex buffers of P = lpt/2 pair rows with a pitch of n + 1 (bank offset
@@ -256,30 +309,8 @@ __global__ void __launch_bounds__(256) k_dct_fft(AxisArgs a)
     if (active) {
         double* ra = out + (size_t)(2 * p) * pitch;
         double* rb = ra + pitch;
-        if (FWD) {
-            // X[k] = Re(e^{-i th_k} V[k]); P = Z[k] + conj(Z[n-k]) = 2 Va[k],
-            // Q = Z[k] - conj(Z[n-k]) = 2i Vb[k]; csh holds (cos, sin)/2
-            for (int k = g; k <= h; k += a.G) {
-                if (k == 0) { ra[0] = z[0].x; rb[0] = z[0].y; continue; }
-                const double2 Zk = z[k], Zm = z[n - k];
-                const double Pr = Zk.x + Zm.x, Pi = Zk.y - Zm.y;
-                const double Qr = Zk.x - Zm.x, Qi = Zk.y + Zm.y;
-                const double2 t = __ldg(a.csh + k);
-                ra[k] = fma(t.x, Pr, t.y * Pi);
-                rb[k] = fma(t.x, Qi, -t.y * Qr);
-                if (k < h) {
-                    ra[n - k] = fma(t.y, Pr, -t.x * Pi);
-                    rb[n - k] = fma(t.y, Qi, t.x * Qr);
-                }
-            }
-        } else {
-            // y = conj(FFT(conj Z)), undone from the reordering
-            for (int i = g; i < n; i += a.G) {
-                const double2 v = z[makhoul_pos(i, n)];
-                ra[i] = v.x;
-                rb[i] = -v.y;
-            }
-        }
+        if (FWD) dct_post(z, ra, rb, n, g, a.G, a.csh);
+        else dct_unpack(z, ra, rb, n, g, a.G);
     }
     __syncthreads();
     for (int e = threadIdx.x; e < tile_elems; e += blockDim.x) {
@@ -443,7 +474,7 @@ struct YzyArgs {
 __global__ void __launch_bounds__(1024) k_dct_yzy(YzyArgs a)
 {
     extern __shared__ double2 smem_all[];
-    const int n = a.n, pitch = n + 1, P = a.pairs, nz = a.nz, nx = a.nx, h = n >> 1;
+    const int n = a.n, pitch = n + 1, P = a.pairs, nz = a.nz, nx = a.nx;
     const int kx = blockIdx.x;
     double2* stw = smem_all;
     double2* sm = smem_all + n;
@@ -474,23 +505,8 @@ __global__ void __launch_bounds__(1024) k_dct_yzy(YzyArgs a)
                                  stw);
     const int c1 = stages & 1;
     double* rows = reinterpret_cast<double*>(sm + (size_t)(c1 ^ 1) * bstride);   // row z at pitch n + 1 doubles
-    if (active) {
-        double* ra = rows + (size_t)(2 * p) * pitch;
-        double* rb = ra + pitch;
-        for (int k = g; k <= h; k += a.G) {
-            if (k == 0) { ra[0] = zf[0].x; rb[0] = zf[0].y; continue; }
-            const double2 Zk = zf[k], Zm = zf[n - k];
-            const double Pr = Zk.x + Zm.x, Pi = Zk.y - Zm.y;
-            const double Qr = Zk.x - Zm.x, Qi = Zk.y + Zm.y;
-            const double2 t = __ldg(a.csh + k);
-            ra[k] = fma(t.x, Pr, t.y * Pi);
-            rb[k] = fma(t.x, Qi, -t.y * Qr);
-            if (k < h) {
-                ra[n - k] = fma(t.y, Pr, -t.x * Pi);
-                rb[n - k] = fma(t.y, Qi, t.x * Qr);
-            }
-        }
-    }
+    double* ra = rows + (size_t)(2 * p) * pitch;
+    if (active) dct_post(zf, ra, ra + pitch, n, g, a.G, a.csh);
     __syncthreads();
     // z: the tridiagonal system of y-mode ky, in place in the real rows
     bool bad = false;
@@ -517,37 +533,107 @@ __global__ void __launch_bounds__(1024) k_dct_yzy(YzyArgs a)
     // inverse along y: the real rows (buffer c1 ^ 1) packed into buffer c1 as in
     // k_dct_fft, then the FFT; a pair writes only its own two rows' storage
     double2* xi = sm + (size_t)c1 * bstride + (size_t)p * pitch;
-    if (active) {
-        const double* ra = rows + (size_t)(2 * p) * pitch;
-        const double* rb = ra + pitch;
-        for (int k = g; k <= h; k += a.G) {
-            if (k == 0) { xi[0] = make_double2(ra[0], -rb[0]); continue; }
-            const double Akx = ra[k], Aky = rb[k], Amx = ra[n - k], Amy = rb[n - k];
-            const double2 t = __ldg(a.cs + k);
-            const double ar = fma(t.x, Akx, t.y * Amx), ai = fma(t.y, Akx, -t.x * Amx);
-            const double br = fma(t.x, Aky, t.y * Amy), bi = fma(t.y, Aky, -t.x * Amy);
-            xi[k] = make_double2(ar - bi, -(ai + br));
-            if (k < h) xi[n - k] = make_double2(ar + bi, ai - br);
-        }
-    }
+    if (active) dct_pack(ra, ra + pitch, xi, n, g, a.G, a.cs);
     pair_sync(a.G);
     const double2* zi = fft_pow2(xi, sm + (size_t)(c1 ^ 1) * bstride + (size_t)p * pitch, n, a.logn, g, a.G, active,
                                  stw);
     const int c2 = (c1 + stages) & 1;
     double* out = reinterpret_cast<double*>(sm + (size_t)(c2 ^ 1) * bstride);
     if (active) {
-        double* ra = out + (size_t)(2 * p) * pitch;
-        double* rb = ra + pitch;
-        for (int i = g; i < n; i += a.G) {
-            const double2 v = zi[makhoul_pos(i, n)];
-            ra[i] = v.x;
-            rb[i] = -v.y;
-        }
+        double* ro = out + (size_t)(2 * p) * pitch;
+        dct_unpack(zi, ro, ro + pitch, n, g, a.G);
     }
     __syncthreads();
     for (int e = threadIdx.x; e < nz * n; e += blockDim.x) {
         const int z = e >> a.logn, y = e & (n - 1);
         a.dst[((size_t)z * n + y) * nx + kx] = out[(size_t)z * pitch + y];
+    }
+}
+
+// The last transformed axis (FFT path) with the spectral division: forward,
+// x_hat times the mode's weight, inverse, one pass over the data where it took
+// three (forward, division, inverse).  The weight is A[p] (the tabulated w/a of the
+// second-order stencil with nz = 1) or w/(1 - g (ex[kx] + ey[ky] + ez[kz])).
+struct SpecArgs {
+    const double* A;                    // null: from the eigenvalues
+    const double *ex, *ey, *ez;
+    int nx, ny;
+    double g, w;
+    int* status;
+    int* iter_log;
+    int* flags;
+};
+
+__global__ void __launch_bounds__(256) k_dct_last(AxisArgs a, SpecArgs c)
+{
+    extern __shared__ double2 smem_all[];
+    const int n = a.n, pitch = n + 1, P = a.lpt >> 1;
+    double2* stw = smem_all;
+    double2* sm = smem_all + n;
+    const size_t bstride = (size_t)P * pitch;
+    __shared__ int base[32];
+    tile_bases(a, blockIdx.x * a.lpt, base);
+    __syncthreads();
+    for (int m = threadIdx.x; m < n; m += blockDim.x) stw[m] = __ldg(a.tw + m);
+    const int tile_elems = a.lpt * n;
+    for (int e = threadIdx.x; e < tile_elems; e += blockDim.x) {
+        int l, i;
+        tile_pos(a, e, l, i);
+        const int b = base[l];
+        double* row = reinterpret_cast<double*>(sm + (size_t)(l >> 1) * pitch);
+        row[2 * makhoul_pos(i, n) + (l & 1)] = b >= 0 ? a.src[b + i * a.inner] : 0.0;
+    }
+    __syncthreads();
+    const int p0 = threadIdx.x / a.G, g = threadIdx.x - p0 * a.G;
+    const bool active = p0 < P;
+    const int p = active ? p0 : 0;
+    const int stages = (a.logn >> 1) + (a.logn & 1), c1 = stages & 1, c2 = (c1 + stages) & 1;
+    const double2* zf = fft_pow2(sm + (size_t)p * pitch, sm + bstride + (size_t)p * pitch, n, a.logn, g, a.G, active,
+                                 stw);
+    double* rows = reinterpret_cast<double*>(sm + (size_t)(c1 ^ 1) * bstride);   // row l at pitch n + 1 doubles
+    double* ra = rows + (size_t)(2 * p) * pitch;
+    if (active) dct_post(zf, ra, ra + pitch, n, g, a.G, a.csh);
+    __syncthreads();
+    bool bad = false;
+    for (int e = threadIdx.x; e < tile_elems; e += blockDim.x) {
+        int l, i;
+        tile_pos(a, e, l, i);
+        const int b = base[l];
+        if (b < 0) continue;
+        const int q = b + i * a.inner;
+        double v = rows[l * pitch + i];
+        if (c.A) {
+            v *= __ldg(c.A + q);
+        } else {
+            const int r = q / c.nx, kx = q - r * c.nx, kz = r / c.ny, ky = r - kz * c.ny;
+            v = c.w * v / (1.0 - c.g * ((c.ex[kx] + c.ey[ky]) + c.ez[kz]));
+        }
+        rows[l * pitch + i] = v;
+        bad |= !isfinite(v);
+    }
+    if (bad) atomicOr(c.flags, ESDC_FLAG_NONFINITE);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        c.status[0] = 1;
+        if (c.iter_log) *c.iter_log = 1;
+    }
+    __syncthreads();
+    // a pair packs its two real rows (buffer c1 ^ 1) into its row of buffer c1
+    double2* xi = sm + (size_t)c1 * bstride + (size_t)p * pitch;
+    if (active) dct_pack(ra, ra + pitch, xi, n, g, a.G, a.cs);
+    pair_sync(a.G);
+    const double2* zi = fft_pow2(xi, sm + (size_t)(c1 ^ 1) * bstride + (size_t)p * pitch, n, a.logn, g, a.G, active,
+                                 stw);
+    double* out = reinterpret_cast<double*>(sm + (size_t)(c2 ^ 1) * bstride);
+    if (active) {
+        double* ro = out + (size_t)(2 * p) * pitch;
+        dct_unpack(zi, ro, ro + pitch, n, g, a.G);
+    }
+    __syncthreads();
+    for (int e = threadIdx.x; e < tile_elems; e += blockDim.x) {
+        int l, i;
+        tile_pos(a, e, l, i);
+        const int b = base[l];
+        if (b >= 0) a.dst[b + i * a.inner] = out[l * pitch + i];
     }
 }
 
@@ -658,7 +744,8 @@ int g_sms = 0;
 // to fill a warp, else ESDC_DCT_MAXPAIRS; a 128-point line pair is one warp,
 // so its stages meet at warp barriers.  Small blocks spread the tiles evenly
 // over the SMs (measured on the 128x128x32 slab: 2 pairs of 128-point lines
-// per block solve 3.8% faster than 8).  Dense path: 128 threads per
+// per block solve 3.8% faster than 8), down to one pair where two would leave SMs
+// without a block (256x256: 64 blocks, now 128).  Dense path: 128 threads per
 // block of up to 32 lines.  Both keep the tile's shared memory below
 // kDctSmemLimit.
 void axis_shape(const DctAxisDev& ax, int lines, AxisArgs& a, int& threads, size_t& smem, int& tiles)
@@ -675,6 +762,7 @@ void axis_shape(const DctAxisDev& ax, int lines, AxisArgs& a, int& threads, size
         if (P < 1) P = 1;
         lpt = 2 * P;
         while (lpt > 2 && (size_t)(lpt * (n + 1) + n) * 16 > (size_t)kDctSmemLimit) lpt >>= 1;
+        while (lpt > 2 && (lpt / 4) * G >= 32 && (lines + lpt - 1) / lpt < g_sms) lpt >>= 1;
         a.G = G;
         threads = (lpt / 2) * G;
         threads = (threads + 31) / 32 * 32;
@@ -719,6 +807,25 @@ cudaError_t axis_pass(const DctAxisDev& ax, bool fwd, const double* src, double*
     return cudaGetLastError();
 }
 
+// The last transformed axis with the spectral division (k_dct_last).
+cudaError_t axis_last(const DctAxisDev& ax, const SpecArgs& c, const double* src, double* dst, int lines, int inner,
+                      cudaStream_t s)
+{
+    AxisArgs a{};
+    int threads;
+    size_t smem;
+    int tiles;
+    axis_shape(ax, lines, a, threads, smem, tiles);
+    a.src = src;
+    a.dst = dst;
+    a.inner = inner;
+    a.tw = ax.tw;
+    a.csh = ax.csh;
+    a.cs = ax.cs;
+    k_dct_last<<<(unsigned)tiles, threads, smem, s>>>(a, c);
+    return cudaGetLastError();
+}
+
 cudaError_t prepare_kernels()
 {
     static bool done = false;
@@ -731,6 +838,8 @@ cudaError_t prepare_kernels()
     if ((e = cudaFuncSetAttribute(k_dct_fft<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) != cudaSuccess)
         return e;
     if ((e = cudaFuncSetAttribute(k_dct_fft<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) != cudaSuccess)
+        return e;
+    if ((e = cudaFuncSetAttribute(k_dct_last, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) != cudaSuccess)
         return e;
     if ((e = cudaFuncSetAttribute(k_dct_dense, cudaFuncAttributeMaxDynamicSharedMemorySize, lim)) != cudaSuccess)
         return e;
@@ -831,8 +940,24 @@ cudaError_t esdc_dct_launch(const MeshDev& m, const CgWork& w, double g, const d
     const double* src = b;
     auto next = [&]() { double* o = bufs[nb]; nb ^= 1; return o; };
     double wgt = 1.0;
+    // The last transformed axis (0 x, 1 y, 2 z) goes forward, through the division and back in one
+    // kernel where it is an FFT axis and nothing else lies between (the second order's z solves do).
+    const int la = m.order == 4 && nz > 1 ? 2 : ny > 1 ? 1 : nx > 1 ? 0 : -1;
+    const DctAxisDev* axs[3] = {&d.ax, &d.ay, &d.az};
+    const bool last = la >= 0 && axs[la]->logn >= 0 && (m.order == 4 || nz == 1);
+    SpecArgs sp{nullptr, d.ex, d.ey, d.ez, nx, ny, g, 0.0, w.status, iter_log, flags};
+    auto spectral = [&]() {
+        double* o = la == 0 || (nx == 1 && (la == 1 || ny == 1)) ? x : next();
+        sp.w = wgt;
+        const int n = la == 0 ? nx : la == 1 ? ny : nz;
+        const cudaError_t err = axis_last(*axs[la], sp, src, o, N / n, la == 0 ? 1 : la == 1 ? nx : sxy, s);
+        src = o;
+        return err;
+    };
     // forward: x, then y (then z for the fourth order)
-    if (nx > 1) {
+    if (nx > 1 && last && la == 0) {
+        wgt /= nx;
+    } else if (nx > 1) {
         double* o = next();
         if ((e = axis_pass(d.ax, true, src, o, N / nx, 1, s)) != cudaSuccess) return e;
         src = o;
@@ -840,7 +965,7 @@ cudaError_t esdc_dct_launch(const MeshDev& m, const CgWork& w, double g, const d
     }
     const bool yzy = m.order == 2 && d.yzy;        // y forward, z, y inverse in k_dct_yzy
     if (ny > 1) {
-        if (!yzy) {
+        if (!yzy && !(last && la == 1)) {
             double* o = next();
             if ((e = axis_pass(d.ay, true, src, o, N / ny, nx, s)) != cudaSuccess) return e;
             src = o;
@@ -867,7 +992,10 @@ cudaError_t esdc_dct_launch(const MeshDev& m, const CgWork& w, double g, const d
         }
         A = d.ztab + (size_t)2 * N * slot;
         C = A + N;
-        if (yzy) {
+        if (last) {
+            sp.A = A;
+            if ((e = spectral()) != cudaSuccess) return e;
+        } else if (yzy) {
             double* o = nx > 1 ? next() : x;
             YzyArgs ya{};
             ya.src = src;
@@ -897,6 +1025,9 @@ cudaError_t esdc_dct_launch(const MeshDev& m, const CgWork& w, double g, const d
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
             src = o;
         }
+    } else if (last) {
+        if (nz > 1) wgt /= nz;
+        if ((e = spectral()) != cudaSuccess) return e;
     } else {
         if (nz > 1) {
             double* o = next();
@@ -921,12 +1052,12 @@ cudaError_t esdc_dct_launch(const MeshDev& m, const CgWork& w, double g, const d
         }
     }
     // inverse: y, then x; the last stage writes x
-    if (ny > 1 && !yzy) {
+    if (ny > 1 && !yzy && !(last && la == 1)) {
         double* o = nx > 1 ? next() : x;
         if ((e = axis_pass(d.ay, false, src, o, N / ny, nx, s)) != cudaSuccess) return e;
         src = o;
     }
-    if (nx > 1) {
+    if (nx > 1 && !(last && la == 0)) {
         if ((e = axis_pass(d.ax, false, src, x, N / nx, 1, s)) != cudaSuccess) return e;
         src = x;
     }
