@@ -601,13 +601,15 @@ cudaError_t esdc_cg_launch(const MeshDev& mesh, const CgWork& w, double g, const
         return esdc_dct_launch(mesh, w, g, b, x, iter_log, flags, s);
     }
     if (solver == 3) solver = 0;                 // the iterative choice of the automatic mode
+    ChebArgs cheb;
+    const bool use_cheb = solver == 0 && g > 0.0 && esdc_cheb_interval(mesh, g, cheb);
+    if (use_cheb && w.cells && mesh.N <= w.cell_nodes)
+        return esdc_small_solve(mesh, w, g, cheb, b, x, tol, maxit, iter_log, flags, s);
     if (esdc_cg4_eligible(mesh, b, x)) {
         CgArgsHost hq{mesh, w, g, b, x, tol, maxit, precond, iter_log, flags};
         if (solver == 0 && g > 0.0 && esdc_cheb_eligible(mesh, b, x)) return esdc_cheb_launch(hq, s);
         return esdc_cg4_launch(hq, false, s);
     }
-    ChebArgs cheb;
-    const bool use_cheb = solver == 0 && g > 0.0 && esdc_cheb_interval(mesh, g, cheb);
     CgArgs a;
     a.m = mesh;
     a.g = g;

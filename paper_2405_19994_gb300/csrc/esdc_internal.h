@@ -154,6 +154,7 @@ struct SmallAxis {
 struct SmallDev {
     void* part = nullptr;            // partial sums' cells [4][SMs]; nullptr: the mesh is not small
     void* cells = nullptr;           // the nodes' exchange cells [2 or 7][N]
+    unsigned long long* tag = nullptr;   // CgWork::cell_tag
     double* mats = nullptr;          // the axes' matrices; nullptr: no dense DCT for this mesh
     double* winv = nullptr;          // [M_max][ld]
     SmallAxis ax[3] = {};
@@ -176,7 +177,18 @@ struct CgWork {
     int max_blocks;
     int threads;
     DctDev* dct = nullptr;          // set when options.solver = 2
+    // exchange cells of the Chebyshev solves of small meshes (esdc_small_solve); nullptr: none
+    void* cells = nullptr;
+    void* cell_part = nullptr;
+    unsigned long long* cell_tag = nullptr;     // the last tag of the solves so far
+    int cell_nodes = 0;             // nodes that the cells hold
+    int sms = 0;
 };
+
+// x = (I - g A)^{-1} b by the Chebyshev semi-iteration c on w.cells (c: esdc_cheb_interval of g).
+struct ChebArgs;
+cudaError_t esdc_small_solve(const MeshDev& m, const CgWork& w, double g, const ChebArgs& c, const double* b, double* x,
+                             double tol, int maxit, int* iter_log, int* flags, cudaStream_t s);
 
 // Whether the DCT solve costs less than an iterative one on this mesh for the
 // given stencil order: every transformed axis (x and y; z for the fourth

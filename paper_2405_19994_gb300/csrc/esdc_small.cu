@@ -40,7 +40,94 @@ bool dct_small(const esdc_handle* h)
     return ops * h->mesh.N / (2.0 * h->sms) <= kSmallDctCycles;
 }
 
+// One Chebyshev solve by itself: the semi-iteration of the one-launch step (small_cheb) on the
+// correction to the guess x, for meshes of up to a node per thread of one 512-thread block per SM.
+// The launch sequences of such meshes (the adjoint's, and those above kSmallNodes) ran k_cheb or
+// k_cheb4, whose iteration is a store, a grid barrier and a load: 86 us per solve of the 256x256
+// field sheet, 48 here (an iteration is bound by the 16 warps' FP64 issue).  Tags go on from
+// launch to launch (the cells need no clearing, so there is no barrier): every block
+// takes the first from device memory, and block 0 moves it on when the solve has ended,
+// after every block has posted a sum under it.
+struct SolveArgs {
+    MeshDev m;
+    int maxit, log_len;
+    double tol2;
+    const double* b;
+    double* x;
+    SmallCell *cells, *part;
+    unsigned long long* tag;
+    unsigned long long stride;       // tags a solve may use
+    unsigned* bar;
+    int *status, *log, *flags;
+    double g[1], inv_theta[1], log_q;
+    double ca[1][ESDC_SMALL_TAB], cb[1][ESDC_SMALL_TAB], qq[1][ESDC_SMALL_TAB];
+};
+
+template <int NB>
+__global__ void __launch_bounds__(512, 1) k_small_solve(const __grid_constant__ SolveArgs s)
+{
+    const MeshDev& m = s.m;
+    const int nb = blockDim.x, tl = threadIdx.x, p = blockIdx.x * nb + tl, N = m.N;
+    const bool has = p < N;
+    const SmallTag tag0 = __ldcg(s.tag);
+    SmallStencil st;
+    small_stencil(m, p, has, has ? node_idx(m, p) : NodeIdx{0, 0, 0}, st);
+    NodeSolve so{0.0, 0.0, 0.0};
+    if (has) {
+        so.b = s.b[p];
+        so.x = s.x[p];
+        double t = 0.0;
+#pragma unroll
+        for (int e = 0; e < NB; ++e)
+            if ((st.mask >> e) & 1u) t = fma(st.cf[e], s.x[st.q[e]] - so.x, t);
+        so.r = fma(s.g[0], t, so.b - so.x);
+    }
+    SmallTag tag = tag0, nred = tag0;
+    SmallWait wt{s.bar, s.flags, false};
+    const bool mute = __ldcg(s.bar + 2) == blockIdx.x + 1;
+    const double e = small_cheb<NB, true>(st, s, N, 0, 0, p, has, tl, nb, so, tag, nred, wt, mute);
+    // every block has posted its first sum, so every neighbour has read its x
+    if (has) s.x[p] = so.x + e;
+    if (blockIdx.x == 0 && tl == 0) *s.tag = tag0 + s.stride;
+}
+
 }  // namespace
+
+cudaError_t esdc_small_solve(const MeshDev& m, const CgWork& w, double g, const ChebArgs& c, const double* b, double* x,
+                             double tol, int maxit, int* iter_log, int* flags, cudaStream_t st)
+{
+    SolveArgs s;
+    s.m = m;
+    s.maxit = maxit;
+    s.log_len = iter_log ? 1 : 0;
+    s.tol2 = tol * tol;
+    s.b = b;
+    s.x = x;
+    s.cells = static_cast<SmallCell*>(w.cells);
+    s.part = static_cast<SmallCell*>(w.cell_part);
+    s.tag = w.cell_tag;
+    s.stride = 2ULL * (unsigned)maxit + 64;
+    s.bar = w.bar;
+    s.status = w.status;
+    s.log = iter_log;
+    s.flags = flags;
+    s.g[0] = g;
+    s.inv_theta[0] = c.inv_theta;
+    s.log_q = c.log_q;
+    double q2 = 1.0;
+    for (int k = 0; k < ESDC_SMALL_TAB; ++k) {
+        s.ca[0][k] = c.ca[k];
+        s.cb[0][k] = c.cb[k];
+        q2 *= c.q * c.q;
+        s.qq[0][k] = 4.0 * q2;
+    }
+    int nodes = 32;
+    while ((m.N + nodes - 1) / nodes > w.sms) nodes *= 2;
+    const void* k = m.order == 4 ? (const void*)k_small_solve<12>
+                  : m.lay ? (const void*)k_small_solve<10> : (const void*)k_small_solve<6>;
+    void* args[] = {&s};
+    return cudaLaunchCooperativeKernel(k, dim3((m.N + nodes - 1) / nodes), dim3(nodes), args, 0, st);
+}
 
 cudaError_t esdc_small_launch_hh(const StepArgs& a, const void* args, int M, int blocks, int threads, size_t smem,
                                  cudaStream_t s)
@@ -63,6 +150,17 @@ cudaError_t esdc_small_prepare(esdc_handle* h)
     cudaError_t e = cudaMalloc(&d.part, sizeof(SmallCell) * 4 * h->sms);
     if (e != cudaSuccess) return e;
     if ((e = cudaMalloc(&d.cells, sizeof(SmallCell) * (dct ? (int)ESDC_SMALL_BUFS : 2) * h->mesh.N)) != cudaSuccess) return e;
+    // tags of the solves start above any that a step's launch uses
+    const unsigned long long tag0 = 1ULL << 40;
+    if ((e = cudaMalloc((void**)&d.tag, sizeof tag0)) != cudaSuccess) return e;
+    if ((e = cudaMemcpy(d.tag, &tag0, sizeof tag0, cudaMemcpyHostToDevice)) != cudaSuccess) return e;
+    if ((e = cudaMemset(d.cells, 0, sizeof(SmallCell) * 2 * h->mesh.N)) != cudaSuccess) return e;
+    if ((e = cudaMemset(d.part, 0, sizeof(SmallCell) * 4 * h->sms)) != cudaSuccess) return e;
+    h->cg.cells = d.cells;
+    h->cg.cell_part = d.part;
+    h->cg.cell_tag = d.tag;
+    h->cg.cell_nodes = h->sms * kSmallNodesField;
+    h->cg.sms = h->sms;
     if (!dct) return cudaSuccess;
     const int n[3] = {h->mesh.nx, h->mesh.ny, h->mesh.nz};
     std::vector<double> mats;
@@ -98,7 +196,7 @@ cudaError_t esdc_small_prepare(esdc_handle* h)
 
 void esdc_small_destroy(SmallDev* d)
 {
-    void* ptrs[] = {d->part, d->cells, d->mats, d->winv};
+    void* ptrs[] = {d->part, d->cells, d->mats, d->winv, d->tag};
     for (void* p : ptrs)
         if (p) cudaFree(p);
     *d = SmallDev{};

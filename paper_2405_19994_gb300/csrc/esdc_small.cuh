@@ -151,10 +151,10 @@ __device__ __forceinline__ void v_sync(int nb)
 // take: waits for every block's.  Reduction n + 2 reuses the cells of n: a block
 // posts n + 1 after it has taken n, and n + 2 after every block has posted n + 1.
 template <int NV>
-__device__ __forceinline__ void sums_post(const double (&v)[NV], const SmallArgs& s, SmallTag n, int tl, int nb)
+__device__ __forceinline__ void sums_post(const double (&v)[NV], SmallCell* part, SmallTag n, int tl, int nb)
 {
     __shared__ double sh[NV][16];
-    SmallCell* cell = s.part + (size_t)(n & 1) * 2 * gridDim.x + blockIdx.x;
+    SmallCell* cell = part + (size_t)(n & 1) * 2 * gridDim.x + blockIdx.x;
     const int lane = tl & 31, w = tl >> 5, nw = nb >> 5;
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
@@ -175,11 +175,12 @@ __device__ __forceinline__ void sums_post(const double (&v)[NV], const SmallArgs
 }
 
 template <int NV>
-__device__ __forceinline__ void sums_take(const SmallArgs& s, SmallTag n, int tl, int nb, double (&tot)[NV], SmallWait& wt)
+__device__ __forceinline__ void sums_take(const SmallCell* part, SmallTag n, int tl, int nb, double (&tot)[NV],
+                                          SmallWait& wt)
 {
     __shared__ double res[2];
     if (tl < 32) {
-        const SmallCell* cell = s.part + (size_t)(n & 1) * 2 * gridDim.x;
+        const SmallCell* cell = part + (size_t)(n & 1) * 2 * gridDim.x;
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
             const SmallCell* c = cell + (size_t)k * gridDim.x;
@@ -278,10 +279,13 @@ __device__ __noinline__ double small_lap(const SmallStencil& st, const SmallCell
 // The solve's correction to the warm start; tag: the last tag this thread's cells
 // carry (the direction of tag t is in buffer t & 1: a thread publishes t + 1 after
 // it has read its neighbours' t, which they published after reading its t - 1).
-template <int NB>
-__device__ __noinline__ double small_cheb(const SmallStencil& st, const SmallArgs& s, int N, int i, int slot, int p,
+// FIRST: the starting residual's sum is asked for before any iteration (a solve by
+// itself may have none to do), not during the first ones.  mute: this block does not
+// post that sum (esdc_debug_barrier).
+template <int NB, bool FIRST = false, class Args = SmallArgs>
+__device__ __noinline__ double small_cheb(const SmallStencil& st, const Args& s, int N, int i, int slot, int p,
                                           bool has, int tl, int nb, const NodeSolve& so, SmallTag& tag, SmallTag& nred,
-                                          SmallWait& wt)
+                                          SmallWait& wt, bool mute = false)
 {
     double cf[NB];
     int q[NB];
@@ -294,13 +298,49 @@ __device__ __noinline__ double small_cheb(const SmallStencil& st, const SmallArg
     if (has) cell_put(s.cells + (tag & 1) * N + p, d, tag);
     {
         const double v[2] = {r * r, has ? so.b * so.b : 0.0};
-        sums_post<2>(v, s, ++nred, tl, nb);
+        ++nred;
+        if (!FIRST || !mute) sums_post<2>(v, s.part, nred, tl, nb);
     }
-    const int first = s.maxit < ESDC_SMALL_MINIT ? s.maxit : ESDC_SMALL_MINIT;
+    const int first = FIRST ? 0 : (s.maxit < ESDC_SMALL_MINIT ? s.maxit : ESDC_SMALL_MINIT);
     int it = 0, check_at = first;
-    double stop = 0.0;
+    double stop = 0.0, tot0 = 0.0;
     bool done = false, bad = false;
-    for (;;) {
+    auto ask = [&]() {
+        // the iterations the bound asks for: the first k with 2 q^k ||r_0|| <= tol ||b||
+        double tot[2];
+        sums_take<2>(s.part, nred, tl, nb, tot, wt);
+        tot0 = tot[0];
+        stop = s.tol2 * tot[1];
+        bad = !isfinite(tot[0]) || !isfinite(stop);
+        __shared__ int s_need;
+        if (tl < 32) {
+            int need = 0;
+            if (!(tot[0] <= stop)) {
+                need = ESDC_SMALL_TAB;
+                for (int k0 = 0; k0 < ESDC_SMALL_TAB; k0 += 32) {
+                    const unsigned hit = __ballot_sync(0xffffffffu, s.qq[i][k0 + tl] * tot[0] <= stop);
+                    if (hit) { need = k0 + __ffs(hit); break; }
+                }
+            }
+            if constexpr (FIRST) {                        // past the table by the formula
+                if (need == ESDC_SMALL_TAB && stop > 0.0) {
+                    const double kd = ceil(log(0.5 * sqrt(stop / tot[0])) / s.log_q);
+                    need = kd < (double)s.maxit ? (int)kd : s.maxit;
+                } else if (need == ESDC_SMALL_TAB) {
+                    need = s.maxit;                       // tol 0: to the cap
+                }
+            }
+            if (tl == 0) s_need = need;
+        }
+        v_sync(nb);
+        check_at = s_need > first ? s_need : first;
+        if (check_at > s.maxit) check_at = s.maxit;
+    };
+    if (FIRST) {
+        ask();
+        done = tot0 <= stop;
+    }
+    while (!FIRST || !(done || bad)) {
         const int ki = it < ESDC_SMALL_TAB ? it : ESDC_SMALL_TAB - 1;
         if (has) {
             double dv[NB];
@@ -316,34 +356,15 @@ __device__ __noinline__ double small_cheb(const SmallStencil& st, const SmallArg
             d = fma(s.ca[i][ki], d, s.cb[i][ki] * r);
         }
         ++it;
-        if (it == first) {
-            // the iterations the bound asks for: the first k with 2 q^k ||r_0|| <= tol ||b||
-            double tot[2];
-            sums_take<2>(s, nred, tl, nb, tot, wt);
-            stop = s.tol2 * tot[1];
-            bad = !isfinite(tot[0]) || !isfinite(stop);
-            __shared__ int s_need;
-            if (tl < 32) {
-                int need = 0;
-                if (!(tot[0] <= stop)) {
-                    need = ESDC_SMALL_TAB;
-                    for (int k0 = 0; k0 < ESDC_SMALL_TAB; k0 += 32) {
-                        const unsigned hit = __ballot_sync(0xffffffffu, s.qq[i][k0 + tl] * tot[0] <= stop);
-                        if (hit) { need = k0 + __ffs(hit); break; }
-                    }
-                }
-                if (tl == 0) s_need = need;
-            }
-            v_sync(nb);
-            check_at = s_need > first ? s_need : first;
-            if (check_at > s.maxit) check_at = s.maxit;
+        if (!FIRST && it == first) {
+            ask();
             if (bad) break;
         }
         if (it == check_at) {
             const double v[1] = {r * r};
             double rr[1];
-            sums_post<1>(v, s, ++nred, tl, nb);
-            sums_take<1>(s, nred, tl, nb, rr, wt);
+            sums_post<1>(v, s.part, ++nred, tl, nb);
+            sums_take<1>(s.part, nred, tl, nb, rr, wt);
             bad = !isfinite(rr[0]);
             done = rr[0] <= stop;
             if (bad || done || it == s.maxit) break;
