@@ -102,21 +102,37 @@ __global__ void k_adj_gates(AdjArgs a)
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < a.m.N; p += gridDim.x * blockDim.x) {
         const double* bYi = a.bY + (int64_t)ii * NS * ld;
         double* bu = a.i == 1 ? a.byn : a.bY + (int64_t)(ii - 1) * NS * ld;
+        // a gate's loads before its stores: in turn, each store held back the next load
+        // (the compiler cannot tell the arrays apart), a chain of 3 (2 M + 4) L2 trips
+#pragma unroll
         for (int g = 0; g < NG; ++g) {
             const int s = 1 + g;
-            const double bw = bYi[s * ld + p];
-            bu[s * ld + p] += bw;
+            const int64_t jm = ii - 1, fi = ((int64_t)ii * NG + g) * ld + p;
+            double S[M], G[M], bG[M], bS[M], g1 = 0.0, gm = 0.0, bphi = 0.0, phi = 0.0;
+            const double bw = bYi[s * ld + p], b0 = bu[s * ld + p];
 #pragma unroll
             for (int j = 0; j < M; ++j) {
-                const int64_t sij = (((int64_t)ii * M + j) * NG + g) * ld + p;
-                a.bGk[((int64_t)j * NS + s) * ld + p] += a.S[sij] * bw;
-                a.bS[sij] += a.Gk[((int64_t)j * NS + s) * ld + p] * bw;
+                const int64_t sij = (((int64_t)ii * M + j) * NG + g) * ld + p, gj = ((int64_t)j * NS + s) * ld + p;
+                S[j] = a.S[sij];
+                bS[j] = a.bS[sij];
+                G[j] = a.Gk[gj];
+                bG[j] = a.bGk[gj];
             }
             if (a.i >= 2) {
-                const int64_t jm = ii - 1;
-                const double dl = a.Gk1[(jm * NS + s) * ld + p] - a.Gk[(jm * NS + s) * ld + p];
-                a.bPHI[((int64_t)ii * NG + g) * ld + p] += dl * bw;
-                a.bdl[g * ld + p] = a.PHI[((int64_t)ii * NG + g) * ld + p] * bw;
+                g1 = a.Gk1[(jm * NS + s) * ld + p];
+                gm = a.Gk[(jm * NS + s) * ld + p];
+                bphi = a.bPHI[fi];
+                phi = a.PHI[fi];
+            }
+            bu[s * ld + p] = b0 + bw;
+#pragma unroll
+            for (int j = 0; j < M; ++j) {
+                a.bGk[((int64_t)j * NS + s) * ld + p] = fma(S[j], bw, bG[j]);
+                a.bS[(((int64_t)ii * M + j) * NG + g) * ld + p] = fma(G[j], bw, bS[j]);
+            }
+            if (a.i >= 2) {
+                a.bPHI[fi] = fma(g1 - gm, bw, bphi);
+                a.bdl[g * ld + p] = phi * bw;
             }
         }
     }
@@ -134,17 +150,20 @@ __global__ void k_adj_rhs(AdjArgs a)
     const double* Vi = a.Yk1 + (int64_t)ii * NS * ld;
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < a.m.N; p += gridDim.x * blockDim.x) {
         double* bu = a.i == 1 ? a.byn : a.bY + (int64_t)(ii - 1) * NS * ld;
-        const double br = a.brhs[p];
-        bu[p] += br;
+        const double br = a.brhs[p], b0 = bu[p], bfi = a.bFIk[(int64_t)ii * ld + p], gs = a.gsig[p];
+        double bG[M];
 #pragma unroll
-        for (int j = 0; j < M; ++j) a.bGk[(int64_t)j * NS * ld + p] += a.dS0[ii][j] * br;
-        a.bdlt0[p] = a.i >= 2 ? a.dtd[a.i] * br : 0.0;
-        a.bFIk[(int64_t)ii * ld + p] -= a.dtd[a.i] * br;
+        for (int j = 0; j < M; ++j) bG[j] = a.bGk[(int64_t)j * NS * ld + p];
         int ix, iy, iz;
         node_xyz(a.m, p, ix, iy, iz);
         double dsig, aw;
         field_terms(a.m, a.brhs, Vi, a.brhs, p, ix, iy, iz, dsig, aw);
-        a.gsig[p] += gam * dsig;                 // F = (I - gam A) V - rhs: dL/dsigma = gam brhs^T dA/dsigma V
+        bu[p] = b0 + br;
+#pragma unroll
+        for (int j = 0; j < M; ++j) a.bGk[(int64_t)j * NS * ld + p] = fma(a.dS0[ii][j], br, bG[j]);
+        a.bdlt0[p] = a.i >= 2 ? a.dtd[a.i] * br : 0.0;
+        a.bFIk[(int64_t)ii * ld + p] = fma(-a.dtd[a.i], br, bfi);
+        a.gsig[p] = fma(gam, dsig, gs);          // F = (I - gam A) V - rhs: dL/dsigma = gam brhs^T dA/dsigma V
     }
 }
 
@@ -169,43 +188,62 @@ __global__ void k_adj_eval(AdjArgs a)
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < a.m.N; p += gridDim.x * blockDim.x) {
         int ix, iy, iz;
         node_xyz(a.m, p, ix, iy, iz);
-        double u[NS];
-        for (int s = 0; s < NS; ++s) u[s] = U[s * ld + p];
+        // every load before the first store (see k_adj_gates)
+        double u[NS], b0[NS], yn[NG], bG1[NS], bG[NS], bdl[NG], Ln[NG], bL[NG], byn[NG];
+        double bdlt0 = 0.0, bfi = 0.0;
+#pragma unroll
+        for (int s = 0; s < NS; ++s) {
+            u[s] = U[s * ld + p];
+            b0[s] = bu[s * ld + p];
+            bG1[s] = a.bGk1[((int64_t)jm * NS + s) * ld + p];
+            bG[s] = quad ? a.bGk[((int64_t)jm * NS + s) * ld + p] : 0.0;
+        }
+#pragma unroll
+        for (int g = 0; g < NG; ++g) {
+            Ln[g] = a.LAMN[(int64_t)g * ld + p];
+            bL[g] = a.bLAM[(int64_t)g * ld + p];
+            yn[g] = a.yn[(1 + g) * ld + p];
+            byn[g] = a.byn[(1 + g) * ld + p];
+            bdl[g] = quad ? a.bdl[g * ld + p] : 0.0;
+        }
+        if (quad) {
+            bdlt0 = a.bdlt0[p];
+            bfi = a.bFIk[(int64_t)jm * ld + p];
+        }
+        const double gs = a.gsig[p], gp0 = a.gpar[p], gp1 = a.gpar[ld + p];
         // FI = D A u_V
         double dsig, aw;
         field_terms(a.m, a.tmp, U, a.tmp, p, ix, iy, iz, dsig, aw);
         double buV = a.D * aw;
-        a.gsig[p] += a.D * dsig;
+        a.gsig[p] = fma(a.D, dsig, gs);
         // f_E = (stim + mI(u)) / C_m enters G_V and dlt0
-        const double bdlt0 = quad ? a.bdlt0[p] : 0.0;
-        const double bmI = (a.bGk1[(int64_t)jm * NS * ld + p] + bdlt0) * a.inv_Cm;
+        const double bmI = (bG1[0] + bdlt0) * a.inv_Cm;
         double dmI[NS], dpar[2];
         HH::currents_d(a.mp.p, u, dmI, dpar);
         buV += dmI[0] * bmI;
         double bus[NS];
         for (int s = 1; s < NS; ++s) bus[s] = dmI[s] * bmI;
-        a.gpar[p] += dpar[0] * bmI;
-        a.gpar[ld + p] += dpar[1] * bmI;
+        a.gpar[p] = fma(dpar[0], bmI, gp0);
+        a.gpar[ld + p] = fma(dpar[1], bmI, gp1);
         if (quad) {                      // dlt0 = fE^{k+1} - (G^k_V - FI^k)
-            a.bGk[(int64_t)jm * NS * ld + p] -= bdlt0;
-            a.bFIk[(int64_t)jm * ld + p] += bdlt0;
+            a.bGk[(int64_t)jm * NS * ld + p] = bG[0] - bdlt0;
+            a.bFIk[(int64_t)jm * ld + p] = bfi + bdlt0;
         }
         // gates: G_g = lam(u_V)(u_g - yinf(u_V)) + Lambda_n (yn_g - u_g); dl_g = G_g - G^k_g
+#pragma unroll
         for (int g = 0; g < NG; ++g) {
             const int s = 1 + g;
             double lam, yinf, dlam, dyinf;
             HH::gate_d(a.mp.p, g, u[0], lam, yinf, dlam, dyinf);
-            const double bdl = quad ? a.bdl[g * ld + p] : 0.0;
-            const double bgn = a.bGk1[((int64_t)jm * NS + s) * ld + p] + bdl;
-            if (quad) a.bGk[((int64_t)jm * NS + s) * ld + p] -= bdl;
-            const double Ln = a.LAMN[(int64_t)g * ld + p];
-            bus[s] += bgn * (lam - Ln);
+            const double bgn = bG1[s] + bdl[g];
+            if (quad) a.bGk[((int64_t)jm * NS + s) * ld + p] = bG[s] - bdl[g];
+            bus[s] += bgn * (lam - Ln[g]);
             buV += bgn * (dlam * (u[s] - yinf) - lam * dyinf);
-            a.bLAM[(int64_t)g * ld + p] += bgn * (a.yn[s * ld + p] - u[s]);
-            a.byn[s * ld + p] += bgn * Ln;
+            a.bLAM[(int64_t)g * ld + p] = fma(bgn, yn[g] - u[s], bL[g]);
+            a.byn[s * ld + p] = fma(bgn, Ln[g], byn[g]);
         }
-        bu[p] += buV;
-        for (int s = 1; s < NS; ++s) bu[s * ld + p] += bus[s];
+        bu[p] = b0[0] + buV;
+        for (int s = 1; s < NS; ++s) bu[s * ld + p] = b0[s] + bus[s];
     }
 }
 
@@ -292,21 +330,25 @@ __global__ void k_gather_sensors(const double* V, const int* sens, double* out, 
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) out[k] = V[sens[k]];
 }
 
-// Deterministic sums of the per-node parameter derivatives (one block, fixed order).
-__global__ void k_sum2(const double* g, int64_t ld, int N, double* out)
+// Deterministic sums of the per-node parameter derivatives: a block per row, four running
+// sums per thread (a load's latency is what bounds it: 256 us for 65,536 nodes with both rows
+// in one block of 256 threads and one sum each), then a fixed tree.
+__global__ void __launch_bounds__(1024) k_sum2(const double* g, int64_t ld, int N, double* out)
 {
-    __shared__ double sh[2][256];
-    for (int r = 0; r < 2; ++r) {
-        double s = 0.0;
-        for (int p = threadIdx.x; p < N; p += blockDim.x) s += g[r * ld + p];
-        sh[r][threadIdx.x] = s;
-    }
+    __shared__ double sh[1024];
+    const double* row = g + blockIdx.x * ld;
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int p = threadIdx.x; p < N; p += 4096)
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (p + 1024 * e < N) s[e] += row[p + 1024 * e];
+    sh[threadIdx.x] = (s[0] + s[1]) + (s[2] + s[3]);
     __syncthreads();
-    if (threadIdx.x < 2) {
-        double s = 0.0;
-        for (int t = 0; t < (int)blockDim.x; ++t) s += sh[threadIdx.x][t];
-        out[threadIdx.x] = s;
+    for (int h = 512; h > 0; h >>= 1) {
+        if ((int)threadIdx.x < h) sh[threadIdx.x] += sh[threadIdx.x + h];
+        __syncthreads();
     }
+    if (threadIdx.x == 0) out[blockIdx.x] = sh[0];
 }
 
 struct AdjWork {
@@ -518,7 +560,7 @@ int esdc_adjoint_backward(esdc_handle* h, const double* ckpt, double t0, double 
         cudaError_t e = reverse_step_M(h, w, a, M, K, s);
         if (e != cudaSuccess) return set_err(h, ESDC_ERR_CUDA, "adjoint step: %s", cudaGetErrorString(e));
     }
-    k_sum2<<<1, 256, 0, s>>>(w.gpar, ld, h->mesh.N, w.sum2);
+    k_sum2<<<2, 1024, 0, s>>>(w.gpar, ld, h->mesh.N, w.sum2);
     CUDA_TRY(h, cudaGetLastError());
     CUDA_TRY(h, cudaMemcpyAsync(gsig, gs, sizeof(double) * h->mesh.N, cudaMemcpyDeviceToDevice, s));
     if (gy0) CUDA_TRY(h, cudaMemcpyAsync(gy0, w.lam, sizeof(double) * NSld, cudaMemcpyDeviceToDevice, s));

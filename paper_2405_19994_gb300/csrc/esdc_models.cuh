@@ -202,26 +202,30 @@ struct HH1952 {
     {
         const double v = V - mp[6];
         auto fprime = [](double x, double f) {
-            return fabs(x) < 1e-3 ? -0.5 + x * (1.0 / 6.0 - x * x * (1.0 / 180.0)) : f * (1.0 - f - x) / x;
+            return fabs(x) < 1e-3 ? -0.5 + x * (1.0 / 6.0 - x * x * (1.0 / 180.0)) : f * (1.0 - f - x) * esdc_rcp(x);
         };
-        double al, be, dal, dbe;
-        rates(q, v, al, be);                       // the forward rates, bit for bit
+        double al, be, dal, dbe;                   // the rates as rates() has them, bit for bit
         if (q == 0) {
+            rates(q, v, al, be);
             dal = -0.1 * fprime((25.0 - v) * 0.1, al);
             dbe = be * (-1.0 / 18.0);
         } else if (q == 1) {
+            rates(q, v, al, be);
             dal = -0.05 * al;
             dbe = 0.1 * be * (1.0 - be);
         } else {
-            const double x = (10.0 - v) * 0.1;
-            dal = 0.1 * (-0.1) * fprime(x, x_over_expm1(x));
+            const double x = (10.0 - v) * 0.1, f = x_over_expm1(x);
+            al = 0.1 * f;
+            be = 0.125 * esdc_exp(v * (-0.0125));
+            dal = 0.1 * (-0.1) * fprime(x, f);
             dbe = be * (-0.0125);
         }
-        const double sum = al + be;
+        // reciprocals of 3 FP64 operations each: an IEEE division is about 9
+        const double sum = al + be, rs = esdc_rcp(sum);
         lam = -sum;
-        yinf = al * esdc_rcp(sum);
+        yinf = al * rs;
         dlam = -(dal + dbe);
-        dyinf = (dal * be - al * dbe) / (sum * sum);
+        dyinf = (dal * be - al * dbe) * (rs * rs);
     }
     // Resting state at V0: gates at w_inf(V0).
     __device__ static void rest(const double* mp, double V0, double* u)
