@@ -825,9 +825,9 @@ __device__ bool cheb_all(const BCgArgs& a, unsigned& target)
 }
 
 // PER_SM: blocks of 512 threads that the registers allow per SM.  One (104 registers, more loads
-// in flight per warp) while a 512-thread block per SM has a warp for every tile, else two (64):
-// 16 slices of 256x256 (2048 tiles) 9.12 / 9.28 ms per Q^par solve, 64 tissues of 64..512 nodes a
-// side (9,900 tiles) 31.4 / 28.5 ms per step.
+// in flight per warp) while a 512-thread block per SM has a warp for every tile, else two (64; or
+// four of 256): 16 slices of 256x256 (2048 tiles) 9.12 / 9.28 ms per Q^par solve, 64 tissues of
+// 64..512 nodes a side (9,900 tiles) 31.4 / 28.5 ms per step.
 template <int PER_SM>
 __global__ void __launch_bounds__(512, PER_SM) k_chebb(BCgArgs a)
 {
@@ -1060,16 +1060,18 @@ int cg_grid(const esdc_batch* b, int threads, int per_sm_wanted)
     return (int)nb;
 }
 
-// The solve's shape until esdc_batch_set_shape gives one: a warp takes whole tiles, so the blocks
-// have as many warps as it takes to give every SM its share of the tiles, 16 at most (then two
-// blocks per SM).  With 512-thread blocks throughout, the 32 tiles of a 128x128 sheet ran on two of
-// the 152 SMs.
+// The solve's shape until esdc_batch_set_shape gives one.  A warp takes whole tiles: one block
+// per SM with as many warps as give every SM its share of the tiles, or, above 16 tiles per SM,
+// four 256-thread blocks per SM (their barriers' waits overlap: 64 tissues of 64..512 nodes a side
+// 27.0 ms per step against 28.4 with two blocks of 512).  With 512-thread blocks throughout, the
+// 32 tiles of a 128x128 sheet ran on two of the 152 SMs.
 void auto_shape(esdc_batch* b)
 {
+    const bool many = b->opt.solver == 0 && many_tiles(b);
     const int warps = std::max(1, std::min(16, (b->ntiles + b->sms - 1) / b->sms));
-    b->cg_threads = 512;
-    b->cg_launch = 32 * warps;
-    b->cg_blocks = cg_grid(b, b->cg_launch, b->opt.solver == 0 && many_tiles(b) ? 2 : 1);
+    b->cg_threads = many ? 256 : 512;
+    b->cg_launch = many ? 256 : 32 * warps;
+    b->cg_blocks = cg_grid(b, b->cg_launch, many ? 4 : 1);
 }
 
 // The step's kernel arguments for M collocation nodes and step dt (the
@@ -1784,7 +1786,7 @@ int esdc_batch_tune(esdc_batch* b, double* y_scratch, double V0, double t, doubl
     // persistent step kernel with its block size and node tile.  None changes
     // a bit of the results.  threads 0: the automatic solve shape.
     struct Shape { int persist, waves, threads, per_sm, tile; };
-    const Shape cand[] = {{0, 1, 0, 0, 0}, {0, 4, 0, 0, 0}, {0, 1, 512, 1, 0}, {0, 2, 512, 1, 0}, {0, 4, 512, 1, 0}, {0, 1, 512, 2, 0},
+    const Shape cand[] = {{0, 1, 0, 0, 0}, {0, 4, 0, 0, 0}, {0, 4, 256, 4, 0}, {0, 1, 512, 1, 0}, {0, 2, 512, 1, 0}, {0, 4, 512, 1, 0}, {0, 1, 512, 2, 0},
                           {0, 2, 512, 2, 0}, {0, 4, 512, 2, 0}, {0, 1, 256, 1, 0},
                           {0, 1, 256, 2, 0}, {0, 2, 256, 2, 0}, {0, 4, 256, 2, 0},
                           {1, 0, 512, 0, 32}, {1, 0, 512, 0, 128}, {1, 0, 512, 0, 512},
