@@ -377,9 +377,11 @@ __device__ __forceinline__ void setup_body(const StepArgs& a, const PhaseArgs& p
 // V row.  i == M+1: only the evaluation at y_M^{k+1}.  Each gate's rate is used
 // as soon as it is computed (its G, Delta and update), which keeps few values live.
 #ifndef ESDC_NODE_MINBLOCKS
-#define ESDC_NODE_MINBLOCKS 6      // 6 x 128 threads per SM: at most 85 registers (SYN19: 80, a
-                                   // 76-byte spill; the kernel waits on memory more than on FP64,
-                                   // and 6 blocks beat 5, 7 and 8 on the headline slab)
+#define ESDC_NODE_MINBLOCKS 7      // 7 x 128 threads per SM: at most 72 registers.  The tables' cubics off
+                                   // the FP64 pipe, the kernel waits on memory and on integer work: 5 / 6 /
+                                   // 7 / 8 blocks take 11.14 / 10.36 / 10.15 / 10.25 ms per step on the 128x128x32
+                                   // SYN19 slab, 4.85 / 4.77 / 4.15 / 4.24 on 90x75x19, 9.09 / 9.00 / 8.72 / 8.75 per
+                                   // Q^par solve of 16 256x256 slices
 #endif
 // TAU: batched kernels may add the FAS correction tau (a.tau, rows 1..M; the
 // recursive form adds tau_i - tau_{i-1}, tau_0 = 0, to every row of node i).
@@ -550,8 +552,8 @@ __device__ __forceinline__ void node_body(const StepArgs& a, const PhaseArgs& ph
 // exactly what the two launches compute.
 __device__ __forceinline__ PhaseArgs next_node1(const StepArgs& a) { return PhaseArgs{1, 0.0, a.Gnew, a.Gnew, nullptr}; }
 
-template <class Model, int M, bool MIXED, bool BATCH>
-__global__ void __launch_bounds__(128, ESDC_NODE_MINBLOCKS) k_node(StepArgs a)
+template <class Model, int M, bool MIXED, bool BATCH, int MINB = ESDC_NODE_MINBLOCKS>
+__global__ void __launch_bounds__(128, MINB) k_node(StepArgs a)
 {
     for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < a.m.N; p += gridDim.x * blockDim.x) {
         if (!BATCH) {
@@ -737,6 +739,9 @@ cudaError_t launch_step_kernels(esdc_handle* h, StepArgs& a, double* y, int K, c
     }
     const int nb_setup = resident_grid(h, occ_setup, T);
     const int nb_node = resident_grid(h, occ_node, T);
+    // Meshes of at most 4 blocks per SM gain nothing from a seventh: 128 registers, no spills
+    // (256x256 SYN19 sheet, M 6: 4.79 -> 4.60 ms per step).
+    const bool few = (h->mesh.N + T - 1) / T <= 4 * h->sms;
     const int nb_res = resident_grid(h, occ_res, T);
     const double g0 = h->D;   // operator scale: (I - dt d_i D L)
     const ColloData* C = &h->col[M - 1];
@@ -776,7 +781,8 @@ cudaError_t launch_step_kernels(esdc_handle* h, StepArgs& a, double* y, int K, c
             a.fuse1 = fuse && i == M + 1 && k + 1 < K;
             if (!(fuse && i == 1)) {
                 prof_begin(h, 1, s);
-                k_node<Model, M, MIXED, false><<<nb_node, T, 0, s>>>(a);
+                if (few) k_node<Model, M, MIXED, false, 4><<<nb_node, T, 0, s>>>(a);
+                else k_node<Model, M, MIXED, false><<<nb_node, T, 0, s>>>(a);
                 prof_end(h, s);
                 if ((e = cudaGetLastError()) != cudaSuccess) return e;
             }
