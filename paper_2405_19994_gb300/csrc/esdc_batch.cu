@@ -176,7 +176,8 @@ struct BCgArgs {
     const double* b;
     double* x;
     double *r, *p, *q, *z;
-    double* part;                // [6][ntiles] tile partials: set-up r.z, r.r, b.b | p.q | r.z, r.r
+    double* part;                // CG: [6][ntiles] tile partials: set-up r.z, r.r, b.b | p.q | r.z, r.r;
+                                 // Chebyshev: [3][kSubs ntiles] r.r, b.b | r.r
     unsigned* bar;
     int* flags;
     int* done_at;                // [ntis] iteration after which the tissue stopped (INT_MAX: running)
@@ -199,9 +200,10 @@ struct BlockTissues {
     long long t0, t1;            // this block's tiles
 };
 
-// Per-tissue totals of nv tile-partial slots for the block's tissues: warp w
+// Per-tissue totals of nv slots of partials (SUBS per tile) for the block's tissues: warp w
 // reduces tissues w, w + nwarps, ...; lane l adds tiles l, l + 32, ... of the
 // tissue in order, then the fixed tree.  tot[k * nv + v] in shared memory.
+template <int SUBS = 1>
 __device__ void tissue_totals(const BCgArgs& a, const BlockTissues& bt, const bool* active, int slot0, int nv,
                               double* tot)
 {
@@ -209,9 +211,9 @@ __device__ void tissue_totals(const BCgArgs& a, const BlockTissues& bt, const bo
     for (int k = w; k < bt.n; k += nw) {
         if (!active[k]) continue;
         const TissueDev* T = a.tis + bt.lo + k;
-        const int t0 = T->tile0, nt = T->ntile;
+        const int t0 = SUBS * T->tile0, nt = SUBS * T->ntile;
         for (int v = 0; v < nv; ++v) {
-            const double* pv = a.part + (size_t)(slot0 + v) * a.ntiles + t0;
+            const double* pv = a.part + (size_t)(slot0 + v) * (SUBS * a.ntiles) + t0;
             double s = 0.0;
             for (int j = lane; j < nt; j += 32) s += __ldcg(pv + j);
             s = warp_tree(s);
@@ -495,10 +497,15 @@ enum : int { kStop = 0, kFp64, kFp32, kDefect, kStart64 };
 constexpr int kRefMinNodes = 16385;      // nodes of a tissue from which it iterates in FP32
 constexpr int kRefMaxOut = 8;            // corrections before the FP64 iterations take over
 constexpr double kFmin2 = 1e-11;         // least reduction (squared) asked of one correction
+// A warp takes pieces of 128 nodes, a quarter of a tile, each with its own partial sums: one warp
+// gets an FP64 instruction through every 64 cycles, so 16 nodes per lane took 5 us per pass where a
+// batch has fewer tiles than the GPU has warps (four of an SM's warps keep its pipe busy).
+constexpr int kSubs = 4, kSubNodes = ESDC_TILE / kSubs;
 
 __device__ bool cheb_all(const BCgArgs& a, unsigned& target)
 {
-    constexpr int U = ESDC_TILE / 32;
+    constexpr int U = kSubNodes / 32;
+    const int nsub = a.ntiles * kSubs;
     __shared__ bool s_chk[kMaxBlockTissues], s_ref[kMaxBlockTissues], s_final[kMaxBlockTissues];
     __shared__ int s_mode[kMaxBlockTissues], s_it[kMaxBlockTissues], s_chunk[kMaxBlockTissues];
     __shared__ int s_first[kMaxBlockTissues], s_out[kMaxBlockTissues];
@@ -513,13 +520,13 @@ __device__ bool cheb_all(const BCgArgs& a, unsigned& target)
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nwb = blockDim.x >> 5;
     const long long nwt = (long long)gridDim.x * nwb;
     BlockTissues bt;
-    bt.t0 = (long long)blockIdx.x * nwb * a.ntiles / nwt;
-    bt.t1 = (long long)(blockIdx.x + 1) * nwb * a.ntiles / nwt;
-    const long long wt0 = ((long long)blockIdx.x * nwb + w) * a.ntiles / nwt;
-    const long long wt1 = ((long long)blockIdx.x * nwb + w + 1) * a.ntiles / nwt;
+    bt.t0 = (long long)blockIdx.x * nwb * nsub / nwt;
+    bt.t1 = (long long)(blockIdx.x + 1) * nwb * nsub / nwt;
+    const long long wt0 = ((long long)blockIdx.x * nwb + w) * nsub / nwt;
+    const long long wt1 = ((long long)blockIdx.x * nwb + w + 1) * nsub / nwt;
     if (bt.t1 > bt.t0) {
-        bt.lo = a.tile_tissue[bt.t0];
-        bt.n = a.tile_tissue[bt.t1 - 1] - bt.lo + 1;
+        bt.lo = a.tile_tissue[bt.t0 / kSubs];
+        bt.n = a.tile_tissue[(bt.t1 - 1) / kSubs] - bt.lo + 1;
     } else {
         bt.lo = 0;
         bt.n = 0;
@@ -547,7 +554,7 @@ __device__ bool cheb_all(const BCgArgs& a, unsigned& target)
         // q / n = umulhi(q, floor(2^32/n)) or one more (0 <= q < 2^31; n = 1: 2^32 - 1)
         s_magx[k] = T->nx > 1 ? (unsigned)(0x100000000ull / (unsigned)T->nx) : 0xffffffffu;
         s_magy[k] = T->ny > 1 ? (unsigned)(0x100000000ull / (unsigned)T->ny) : 0xffffffffu;
-        if (T->tile0 >= bt.t0 && T->tile0 < bt.t1) a.done_at[bt.lo + k] = INT_MAX;
+        if (kSubs * T->tile0 >= bt.t0 && kSubs * T->tile0 < bt.t1) a.done_at[bt.lo + k] = INT_MAX;
     }
     __syncthreads();
 
@@ -580,11 +587,11 @@ __device__ bool cheb_all(const BCgArgs& a, unsigned& target)
         return fma(s_diag[k][c], widen(__ldcg(v + q)), -(s_gih2[k] * s));
     };
     auto tile_geo = [&](long long t, int& k) -> TileGeo {
-        const int b = a.tile_tissue[t];
+        const int b = a.tile_tissue[t / kSubs];
         k = b - bt.lo;
         const TissueDev* T = a.tis + b;
         TileGeo G;
-        G.base = (int)(t << ESDC_TILE_SHIFT);
+        G.base = 0;
         G.nx = T->nx; G.ny = T->ny; G.nz = T->nz; G.N = T->N; G.off = T->off;
         return G;
     };
@@ -598,7 +605,7 @@ __device__ bool cheb_all(const BCgArgs& a, unsigned& target)
     auto stop_tissue = [&](int k, int f) {
         s_mode[k] = kStop;
         const TissueDev* T = a.tis + bt.lo + k;
-        if (T->tile0 >= bt.t0 && T->tile0 < bt.t1) {
+        if (kSubs * T->tile0 >= bt.t0 && kSubs * T->tile0 < bt.t1) {
             a.done_at[bt.lo + k] = tick;
             a.status[2 * (bt.lo + k)] = s_it[k];
             a.status[2 * (bt.lo + k) + 1] = f;
@@ -635,10 +642,13 @@ __device__ bool cheb_all(const BCgArgs& a, unsigned& target)
         return rr > 1e-26 * n && rr < 1e26 * n;
     };
 
-    // [S] r = b - B x, d_0 = r / theta; tile partials r.r, b.b (slots 0-1)
+    // [S] r = b - B x, d_0 = r / theta; partials r.r, b.b (slots 0-1)
+    int k = 0;                        // the tile at hand (looked up once for its pieces) and its tissue
+    TileGeo G{};
+    long long at = -1;
     for (long long t = wt0; t < wt1; ++t) {
-        int k;
-        const TileGeo G = tile_geo(t, k);
+        if (t / kSubs != at) { at = t / kSubs; G = tile_geo(t, k); }
+        G.base = (int)t * kSubNodes;
         const double inv_theta = s_itheta[k];
         const bool ref = s_ref[k];
         float* df = reinterpret_cast<float*>(a.p + G.off);
@@ -665,11 +675,11 @@ __device__ bool cheb_all(const BCgArgs& a, unsigned& target)
         v0 = warp_tree(v0); v1 = warp_tree(v1);
         if (lane == 0) {
             a.part[t] = v0;
-            a.part[(size_t)a.ntiles + t] = v1;
+            a.part[(size_t)nsub + t] = v1;
         }
     }
     if (!grid_barrier(a.bar, target, a.flags)) return false;
-    tissue_totals(a, bt, s_chk, 0, 2, s_tot);
+    tissue_totals<kSubs>(a, bt, s_chk, 0, 2, s_tot);
     for (int k = threadIdx.x; k < bt.n; k += blockDim.x) {
         const double rr = s_tot[2 * k], stop = a.tol2 * s_tot[2 * k + 1];
         s_stop[k] = stop;
@@ -702,24 +712,39 @@ __device__ bool cheb_all(const BCgArgs& a, unsigned& target)
             s_chk[k] = s_it[k] + 1 >= s_chunk[k] || s_it[k] + 1 >= a.maxit;
         }
         __syncthreads();
-        // [U] the tissue's pass; tile partials r.r of the checking tissues (slot 2)
+        // [U] the tissue's pass; partials r.r of the checking tissues (slot 2)
         double* dc = odd ? a.q : a.p;
         double* dn = odd ? a.p : a.q;
-        for (long long t = wt0; t < wt1; ++t) {
-            int k;
+        for (long long t = wt0; t < wt1;) {
             const TileGeo G = tile_geo(t, k);
+            const long long t1 = (t / kSubs + 1) * kSubs < wt1 ? (t / kSubs + 1) * kSubs : wt1;   // this tile's pieces
             const int mode = s_mode[k];
-            if (mode == kStop) continue;
             const bool chk = s_chk[k];
-            const int q0 = G.base - G.off + lane;
-            double v = 0.0;
+            const int q0 = (int)t * kSubNodes - G.off + lane;
+            // body(q, v) for the nodes of the pieces t .. t1-1, and their partials (v from zero)
+            auto pieces = [&](auto zero, auto body) {
+                int q = q0;
+                for (long long e = t; e < t1; ++e, q += kSubNodes) {
+                    auto v = zero;
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
+                        if (q + 32 * u < G.N) body(q + 32 * u, v);
+                    if (chk) {
+                        const double sum = warp_tree(v);
+                        if (lane == 0) a.part[2 * (size_t)nsub + e] = sum;
+                    }
+                }
+            };
+            float* df = reinterpret_cast<float*>(a.p + G.off);
+            float* ef = reinterpret_cast<float*>(a.z + G.off);
+            float* zf = ef + pad(G);
+            float* dcf = odd ? df + pad(G) : df;
+            float* dnf = odd ? df : df + pad(G);
             if (mode == kFp64) {
                 // x += d, r -= B d, d' = ca d + cb r
                 const double ca = s_ca[k], cb = s_cb[k];
-#pragma unroll 4
-                for (int u = 0; u < U; ++u) {
-                    const int q = q0 + 32 * u, p = G.off + q;
-                    if (q >= G.N) continue;
+                pieces(0.0, [&](int q, double& v) {
+                    const int p = G.off + q;
                     const double dp = __ldcg(dc + p);
                     const double bd = op(dc + G.off, dp, q, G, k);
                     const double rp = __ldcg(a.r + p) - bd;
@@ -727,61 +752,44 @@ __device__ bool cheb_all(const BCgArgs& a, unsigned& target)
                     a.r[p] = rp;
                     dn[p] = fma(ca, dp, cb * rp);
                     if (chk) v = fma(rp, rp, v);
-                }
+                });
             } else if (mode == kStart64) {
                 const double inv_theta = s_itheta[k];
-                for (int q = q0; q < q0 + ESDC_TILE && q < G.N; q += 32) dn[G.off + q] = __ldcg(a.r + G.off + q) * inv_theta;
-            } else {
-                float* df = reinterpret_cast<float*>(a.p + G.off);
-                float* ef = reinterpret_cast<float*>(a.z + G.off);
-                float* zf = ef + pad(G);
-                float* dcf = odd ? df + pad(G) : df;
-                float* dnf = odd ? df : df + pad(G);
-                if (mode == kFp32) {
-                    // e += d, r -= B d, d' = ca d + cb r; the last one adds e to x
-                    const float ca = (float)s_ca[k], cb = (float)s_cb[k], gf = (float)s_gih2[k];
-                    const bool first = s_it[k] == s_first[k];
-                    float acc = 0.0f;
-#pragma unroll 4
-                    for (int u = 0; u < U; ++u) {
-                        const int q = q0 + 32 * u;
-                        if (q >= G.N) continue;
-                        float s;
-                        const int c = neighbours([&](int j) { return dcf[j]; }, q, G, k, s);
-                        const float d = dcf[q];
-                        const float rn = zf[q] - fmaf(fmaf(gf, (float)c, 1.0f), d, -(gf * s));
-                        const float en = first ? d : ef[q] + d;
-                        ef[q] = en;
-                        if (chk) {
-                            const double xp = a.x[G.off + q];
-                            a.x[G.off + q] = xp + widen(en);
-                            acc = fmaf(rn, rn, acc);
-                        } else {
-                            zf[q] = rn;
-                            dnf[q] = fmaf(ca, d, cb * rn);
-                        }
+                pieces(0.0, [&](int q, double&) { dn[G.off + q] = __ldcg(a.r + G.off + q) * inv_theta; });
+            } else if (mode == kFp32) {
+                // e += d, r -= B d, d' = ca d + cb r; the last one adds e to x
+                const float ca = (float)s_ca[k], cb = (float)s_cb[k], gf = (float)s_gih2[k];
+                const bool first = s_it[k] == s_first[k];
+                pieces(0.0f, [&](int q, float& v) {
+                    float s;
+                    const int c = neighbours([&](int j) { return dcf[j]; }, q, G, k, s);
+                    const float d = dcf[q];
+                    const float rn = zf[q] - fmaf(fmaf(gf, (float)c, 1.0f), d, -(gf * s));
+                    const float en = first ? d : ef[q] + d;
+                    ef[q] = en;
+                    if (chk) {
+                        const double xp = a.x[G.off + q];
+                        a.x[G.off + q] = xp + widen(en);
+                        v = fmaf(rn, rn, v);
+                    } else {
+                        zf[q] = rn;
+                        dnf[q] = fmaf(ca, d, cb * rn);
                     }
-                    v = acc;
-                } else {
-                    // kDefect: r -= B e in FP64, and the next correction's start
-                    const float inv_theta = (float)s_itheta[k];
-#pragma unroll 4
-                    for (int u = 0; u < U; ++u) {
-                        const int q = q0 + 32 * u, p = G.off + q;
-                        if (q >= G.N) continue;
-                        const double rp = __ldcg(a.r + p) - op_wide(ef, q, G, k);
-                        a.r[p] = rp;
-                        const float rf = (float)rp;
-                        zf[q] = rf;
-                        dnf[q] = rf * inv_theta;
-                        v = fma(rp, rp, v);
-                    }
-                }
+                });
+            } else if (mode == kDefect) {
+                // r -= B e in FP64, and the next correction's start
+                const float inv_theta = (float)s_itheta[k];
+                pieces(0.0, [&](int q, double& v) {
+                    const int p = G.off + q;
+                    const double rp = __ldcg(a.r + p) - op_wide(ef, q, G, k);
+                    a.r[p] = rp;
+                    const float rf = (float)rp;
+                    zf[q] = rf;
+                    dnf[q] = rf * inv_theta;
+                    v = fma(rp, rp, v);
+                });
             }
-            if (chk) {
-                v = warp_tree(v);
-                if (lane == 0) a.part[2 * (size_t)a.ntiles + t] = v;
-            }
+            t = t1;
         }
         odd = !odd;
         if (!grid_barrier(a.bar, target, a.flags)) return false;
@@ -794,7 +802,7 @@ __device__ bool cheb_all(const BCgArgs& a, unsigned& target)
         }
         __syncthreads();
         if (s_exit) break;
-        tissue_totals(a, bt, s_chk, 2, 1, s_tot);
+        tissue_totals<kSubs>(a, bt, s_chk, 2, 1, s_tot);
         for (int k = threadIdx.x; k < bt.n; k += blockDim.x) {
             const int mode = s_mode[k];
             if (mode == kStart64) { start64(k); continue; }
@@ -1025,19 +1033,22 @@ int grid_nodes(const esdc_batch* b, int occ, int waves)
     return (int)std::max(1LL, std::min(cap, need));
 }
 
-// Largest number of tissues one CG block touches for a grid of nb blocks.
+// Pieces of a tile that the solve's warps take one by one.
+int solve_subs(const esdc_batch* b) { return b->opt.solver == 0 ? kSubs : 1; }
+
+// Largest number of tissues one solve block touches for a grid of nb blocks.
 int max_block_tissues(const esdc_batch* b, int nb, int threads)
 {
-    const int nwb = threads / 32;
-    const long long nwt = (long long)nb * nwb;
+    const int nwb = threads / 32, subs = solve_subs(b);
+    const long long nwt = (long long)nb * nwb, n = (long long)subs * b->ntiles;
     int worst = 0;
     for (int blk = 0; blk < nb; ++blk) {
-        const long long t0 = (long long)blk * nwb * b->ntiles / nwt, t1 = (long long)(blk + 1) * nwb * b->ntiles / nwt;
+        const long long t0 = (long long)blk * nwb * n / nwt, t1 = (long long)(blk + 1) * nwb * n / nwt;
         if (t1 <= t0) continue;
         int lo = 0, hi = 0;
         for (int k = 0; k < b->ntis; ++k) {                // tissues are in tile order
-            if (b->tis_h[k].tile0 <= t0) lo = k;
-            if (b->tis_h[k].tile0 <= t1 - 1) hi = k;
+            if ((long long)subs * b->tis_h[k].tile0 <= t0) lo = k;
+            if ((long long)subs * b->tis_h[k].tile0 <= t1 - 1) hi = k;
         }
         worst = std::max(worst, hi - lo + 1);
     }
@@ -1054,21 +1065,21 @@ int cg_grid(const esdc_batch* b, int threads, int per_sm_wanted)
     if (occ < 1) return 0;
     int per_sm = std::min(occ, per_sm_wanted);
     long long nb = (long long)b->sms * per_sm;
-    const long long need = ((long long)b->ntiles + threads / 32 - 1) / (threads / 32);
+    const long long need = ((long long)solve_subs(b) * b->ntiles + threads / 32 - 1) / (threads / 32);
     nb = std::max(1LL, std::min(nb, need));
     while (nb > 1 && max_block_tissues(b, (int)nb, threads) > kMaxBlockTissues) --nb;
     return (int)nb;
 }
 
-// The solve's shape until esdc_batch_set_shape gives one.  A warp takes whole tiles: one block
-// per SM with as many warps as give every SM its share of the tiles, or, above 16 tiles per SM,
-// four 256-thread blocks per SM (their barriers' waits overlap: 64 tissues of 64..512 nodes a side
-// 27.0 ms per step against 28.4 with two blocks of 512).  With 512-thread blocks throughout, the
-// 32 tiles of a 128x128 sheet ran on two of the 152 SMs.
+// The solve's shape until esdc_batch_set_shape gives one.  A warp takes whole pieces of tiles: one
+// block per SM with as many warps as give every SM its share, or, above 16 tiles per SM, four
+// 256-thread blocks per SM (their barriers' waits overlap: 64 tissues of 64..512 nodes a side 27.0
+// ms per step against 28.4 with two blocks of 512).  With 512-thread blocks throughout, the 32
+// tiles of a 128x128 sheet ran on two of the 152 SMs.
 void auto_shape(esdc_batch* b)
 {
     const bool many = b->opt.solver == 0 && many_tiles(b);
-    const int warps = std::max(1, std::min(16, (b->ntiles + b->sms - 1) / b->sms));
+    const int warps = (int)std::max(1LL, std::min(16LL, ((long long)solve_subs(b) * b->ntiles + b->sms - 1) / b->sms));
     b->cg_threads = many ? 256 : 512;
     b->cg_launch = many ? 256 : 32 * warps;
     b->cg_blocks = cg_grid(b, b->cg_launch, many ? 4 : 1);
@@ -1139,7 +1150,7 @@ int bstep_grid(const esdc_batch* b, int M)
     const int occ = b->occ_bstep[M][b->p_threads == 256 ? 0 : 1];
     if (occ < 1) return 0;
     long long nb = (long long)b->sms * std::min(occ, b->p_threads == 256 ? 2 : 1);
-    const long long need = ((long long)b->ntiles + b->p_threads / 32 - 1) / (b->p_threads / 32);
+    const long long need = ((long long)solve_subs(b) * b->ntiles + b->p_threads / 32 - 1) / (b->p_threads / 32);
     nb = std::max(1LL, std::min(nb, need));
     while (nb > 1 && max_block_tissues(b, (int)nb, b->p_threads) > kMaxBlockTissues) --nb;
     return (int)nb;
@@ -1503,7 +1514,8 @@ int esdc_batch_create(int n, const esdc_mesh* meshes, const double* sigma, doubl
     struct { double** p; int64_t n; } bufs[] = {
         {&b->Y, Mx * NS * ld}, {&b->G0, Mx * NS * ld}, {&b->G1, Mx * NS * ld}, {&b->FI, Mx * ld},
         {&b->S, Mx * Mx * NG * ld}, {&b->PHI, Mx * NG * ld}, {&b->LAMN, NG * ld}, {&b->rhs, ld},
-        {&b->Vprev, ld}, {&b->r, ld}, {&b->p, ld}, {&b->q, ld}, {&b->z, ld}, {&b->part, 6LL * tile}};
+        {&b->Vprev, ld}, {&b->r, ld}, {&b->p, ld}, {&b->q, ld}, {&b->z, ld}, {&b->part, 3LL * kSubs * tile}};          // the CG's 6 tile partials fit
+    static_assert(3 * kSubs >= 6, "partial sums of either solve");
     for (auto& bf : bufs) {
         cudaError_t e = cudaMalloc((void**)bf.p, sizeof(double) * bf.n);
         if (e != cudaSuccess) return fail(e == cudaErrorMemoryAllocation ? ESDC_ERR_NO_MEMORY : ESDC_ERR_CUDA);
