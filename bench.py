@@ -400,8 +400,8 @@ def run_ours(args):
         roof["classes"] = classes
         roof["classes_note"] = (
             "fp64_issue_frac: FP64 instructions (DFMA, DADD, DMUL; counted by ncu per node, profiles/) per second "
-            "over the FP64 issue peak, 152 SMs x 2 per clock x 2.07 GHz.  On this GPU no class but the "
-            "set-up comes near HBM's rate, the diffusion solve included: the solve's vectors stay in L2, so its GB/s is "
+            "over the FP64 issue peak, 152 SMs x 2 per clock x 2.07 GHz.  On this GPU no class, the "
+            "diffusion solve included, is bound by HBM alone: the solve's vectors stay in L2, so its GB/s is "
             "reported against HBM for reference only (the 70%-of-HBM target assumes an HBM-bound stencil).")
 
     # ---- CPU oracle baseline on one full-size step from the live state (rank 0, N = 1)
