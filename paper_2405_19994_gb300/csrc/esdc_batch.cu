@@ -177,7 +177,7 @@ struct BCgArgs {
     double* x;
     double *r, *p, *q, *z;
     double* part;                // CG: [6][ntiles] tile partials: set-up r.z, r.r, b.b | p.q | r.z, r.r;
-                                 // Chebyshev: [3][kSubs ntiles] r.r, b.b | r.r
+                                 // Chebyshev: [4][kSubs ntiles] r.r, b.b | r.r of even and of odd passes
     unsigned* bar;
     int* flags;
     int* done_at;                // [ntis] iteration after which the tissue stopped (INT_MAX: running)
@@ -712,7 +712,10 @@ __device__ bool cheb_all(const BCgArgs& a, unsigned& target)
             s_chk[k] = s_it[k] + 1 >= s_chunk[k] || s_it[k] + 1 >= a.maxit;
         }
         __syncthreads();
-        // [U] the tissue's pass; partials r.r of the checking tissues (slot 2)
+        // [U] the tissue's pass; partials r.r of the checking tissues, in two slots by turns: a tissue may
+        // check in consecutive passes (a correction, then its defect), and a block that is ahead writes
+        // this pass's partials while another still adds up the last one's
+        const int slot = 2 + (tick & 1);
         double* dc = odd ? a.q : a.p;
         double* dn = odd ? a.p : a.q;
         for (long long t = wt0; t < wt1;) {
@@ -731,7 +734,7 @@ __device__ bool cheb_all(const BCgArgs& a, unsigned& target)
                         if (q + 32 * u < G.N) body(q + 32 * u, v);
                     if (chk) {
                         const double sum = warp_tree(v);
-                        if (lane == 0) a.part[2 * (size_t)nsub + e] = sum;
+                        if (lane == 0) a.part[slot * (size_t)nsub + e] = sum;
                     }
                 }
             };
@@ -802,7 +805,7 @@ __device__ bool cheb_all(const BCgArgs& a, unsigned& target)
         }
         __syncthreads();
         if (s_exit) break;
-        tissue_totals<kSubs>(a, bt, s_chk, 2, 1, s_tot);
+        tissue_totals<kSubs>(a, bt, s_chk, slot, 1, s_tot);
         for (int k = threadIdx.x; k < bt.n; k += blockDim.x) {
             const int mode = s_mode[k];
             if (mode == kStart64) { start64(k); continue; }
@@ -1514,8 +1517,8 @@ int esdc_batch_create(int n, const esdc_mesh* meshes, const double* sigma, doubl
     struct { double** p; int64_t n; } bufs[] = {
         {&b->Y, Mx * NS * ld}, {&b->G0, Mx * NS * ld}, {&b->G1, Mx * NS * ld}, {&b->FI, Mx * ld},
         {&b->S, Mx * Mx * NG * ld}, {&b->PHI, Mx * NG * ld}, {&b->LAMN, NG * ld}, {&b->rhs, ld},
-        {&b->Vprev, ld}, {&b->r, ld}, {&b->p, ld}, {&b->q, ld}, {&b->z, ld}, {&b->part, 3LL * kSubs * tile}};          // the CG's 6 tile partials fit
-    static_assert(3 * kSubs >= 6, "partial sums of either solve");
+        {&b->Vprev, ld}, {&b->r, ld}, {&b->p, ld}, {&b->q, ld}, {&b->z, ld}, {&b->part, 4LL * kSubs * tile}};          // the CG's 6 tile partials fit
+    static_assert(4 * kSubs >= 6, "partial sums of either solve");
     for (auto& bf : bufs) {
         cudaError_t e = cudaMalloc((void**)bf.p, sizeof(double) * bf.n);
         if (e != cudaSuccess) return fail(e == cudaErrorMemoryAllocation ? ESDC_ERR_NO_MEMORY : ESDC_ERR_CUDA);
