@@ -695,7 +695,7 @@ __device__ bool cheb_all(const BCgArgs& a, unsigned& target)
     __syncthreads();
 
     for (tick = 0;; ++tick) {
-        if (tick > a.maxit + kRefMaxOut + 1) {                // cannot happen: every tissue stops by maxit
+        if (tick - (kRefMaxOut + 1) > a.maxit) {              // cannot happen: every tissue stops by maxit
             if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(a.flags, ESDC_FLAG_CG_MAXIT);
             break;
         }

@@ -433,20 +433,20 @@ __device__ bool cheb4_iterate(const CgArgs& a, const ChebArgs& c, const Tab<doub
     double* dc = a.p;            // d_k
     double* dn = a.q;            // d_{k+1}
     __shared__ double bs[1];
+    const int it0 = it, left = a.maxit - it0;
     // iterations the bound asks for: 2 q^k ||r_0|| <= tol ||b||.  One thread per block
     // evaluates it (a few dozen FP64 operations) and shares it; every block gets the same value.
     __shared__ int s_kneed;
     if (threadIdx.x == 0) {
         int kn = 1;
         if (!done && !bad && c.q > 0.0) {
-            const double kd = stop > 0.0 ? ceil(log(0.5 * sqrt(stop / rr0)) / c.log_q) : (double)a.maxit;
-            kn = kd < (double)a.maxit ? (int)kd : a.maxit;     // tol 0: run to the cap
+            const double kd = stop > 0.0 ? ceil(log(0.5 * sqrt(stop / rr0)) / c.log_q) : (double)left;
+            kn = kd < (double)left ? (int)kd : left;           // tol 0: run to the cap
         }
         s_kneed = kn < 1 ? 1 : kn;
     }
     __syncthreads();
-    const int it0 = it;
-    int chunk_end = it0 + s_kneed < a.maxit ? it0 + s_kneed : a.maxit;
+    int chunk_end = it0 + (s_kneed < left ? s_kneed : left);
     while (!done && !bad && it < a.maxit) {
         const bool check = it + 1 >= chunk_end;
         const int k = it - it0, ki = k < ESDC_CHEB_TAB ? k : ESDC_CHEB_TAB - 1;

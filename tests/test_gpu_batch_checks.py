@@ -77,3 +77,14 @@ def test_consecutive_checks(stiff):
         # 12 solves to 1e-14 ||b|| in either run; the explicit terms' factor kappa - 1 is below 1 here
         err = np.linalg.norm(first[k][0] - want[k][0]) / np.linalg.norm(want[k][0])
         assert err <= 12 * 2e-14 * 2.0, (MESHES[k], err)
+
+
+@pytest.mark.parametrize("cap", [2**31 - 1, 2**31 - 9])
+def test_largest_iteration_caps(cap):
+    # cg_maxit is any int from 1 on: the largest ones change nothing
+    wls = tissues(1.0)
+    want, it = run(wls)[0]
+    for persistent in (None, (512, 128)):
+        got, it_n = run(wls, persistent=persistent, cg_maxit=cap)[0]
+        assert it.min() >= 1 and np.array_equal(it, it_n)
+        assert all(np.array_equal(a, b) for a, b in zip(got, want))
