@@ -663,7 +663,13 @@ __global__ void __launch_bounds__(512, 1) k_small_step(const __grid_constant__ S
                     }
                 }
             }
-            if (i > M) break;
+            if (i > M) {
+                // With one node y_M is y_1: the gates' warps may write node 1 of the next sweep only after
+                // the V warps have read y_1 for this evaluation.  (With more nodes that is another row, and
+                // the barrier after its solve orders the rest.)
+                if (M == 1 && k + 1 < s.K) __syncthreads();
+                break;
+            }
             if (role == 0) {
                 double e;
                 if (s.dct) e = small_dct(m, s, i, slot, p, has, tl, nb, so.r, mats, work, wt);
