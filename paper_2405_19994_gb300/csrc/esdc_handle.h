@@ -101,6 +101,9 @@ void esdc_small_destroy(SmallDev* d);
 cudaError_t esdc_small_step(esdc_handle* h, StepArgs& a, double* y, int M, int K, cudaStream_t s, bool* taken);
 cudaError_t esdc_small_launch_hh(const StepArgs& a, const void* args, int M, int blocks, int threads, size_t smem,
                                  cudaStream_t s);
+// Constants of the SYN19 kernels' translation unit on the current device.  At creation: a step may be the first
+// work of its handle inside a stream capture, where a copy to the device is an error.
+cudaError_t esdc_small_constants_syn(int device);
 cudaError_t esdc_small_launch_syn(const StepArgs& a, const void* args, int M, int blocks, int threads, size_t smem,
                                   cudaStream_t s);
 // (Re)builds the handle's gate table for its current parameters (esdc_step.cu).

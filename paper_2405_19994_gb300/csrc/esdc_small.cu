@@ -141,13 +141,16 @@ cudaError_t esdc_small_prepare(esdc_handle* h)
     d = SmallDev{};
     if (h->opt.precision != 0 || h->opt.solver == 1 || (long long)h->mesh.N > (long long)h->sms * kSmallNodesField)
         return cudaSuccess;
-    {
+    cudaError_t e;
+    if (h->model == ESDC_MODEL_HH1952) {
         std::lock_guard<std::mutex> lk(g_const_mu);
-        const cudaError_t e = upload_constants_local(g_const_done, h->device);
-        if (e != cudaSuccess) return e;
+        e = upload_constants_local(g_const_done, h->device);
+    } else {
+        e = esdc_small_constants_syn(h->device);
     }
+    if (e != cudaSuccess) return e;
     const bool dct = h->cg.dct && dct_small(h);
-    cudaError_t e = cudaMalloc(&d.part, sizeof(SmallCell) * 4 * h->sms);
+    e = cudaMalloc(&d.part, sizeof(SmallCell) * 4 * h->sms);
     if (e != cudaSuccess) return e;
     if ((e = cudaMalloc(&d.cells, sizeof(SmallCell) * (dct ? (int)ESDC_SMALL_BUFS : 2) * h->mesh.N)) != cudaSuccess) return e;
     // tags of the solves start above any that a step's launch uses

@@ -8,15 +8,14 @@ std::mutex g_const_mu;
 bool g_const_done[64] = {false};
 }
 
+cudaError_t esdc_small_constants_syn(int device)
+{
+    std::lock_guard<std::mutex> lk(g_const_mu);
+    return upload_constants_local(g_const_done, device);
+}
+
 cudaError_t esdc_small_launch_syn(const StepArgs& a, const void* args, int M, int blocks, int threads, size_t smem,
                                   cudaStream_t s)
 {
-    {
-        std::lock_guard<std::mutex> lk(g_const_mu);
-        int dev = 0;
-        cudaError_t e = cudaGetDevice(&dev);
-        if (e == cudaSuccess) e = upload_constants_local(g_const_done, dev);
-        if (e != cudaSuccess) return e;
-    }
     return small_launch_M<esdc::SYN19>(a, *static_cast<const SmallArgs*>(args), M, blocks, threads, smem, s);
 }
