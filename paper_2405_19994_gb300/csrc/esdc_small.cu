@@ -22,7 +22,6 @@ constexpr int kSmallNodes = 256, kSmallNodesField = 512;
 constexpr double kSmallDctCycles = 40000.0;
 constexpr int kSmallDctAxis = 256;
 constexpr int kSmallDctCable = 128;         // 1D: one line means one block
-constexpr int kSmallStageDoubles = 18 * 1024;
 
 bool dct_small(const esdc_handle* h)
 {

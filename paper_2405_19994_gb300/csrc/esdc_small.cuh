@@ -37,11 +37,14 @@
 // Every wait is bounded (1 s, or esdc_debug_barrier's limit): a thread whose wait
 // runs out raises TIMEOUT and waits for nothing more, so the launch ends.
 #pragma once
+#include <atomic>
+
 #include "esdc_cg_common.cuh"
 #include "esdc_kernels.cuh"
 
 #define ESDC_SMALL_TAB 64
 #define ESDC_SMALL_MINIT 3           // iterations that run before the starting residual's sum is asked for
+constexpr int kSmallStageDoubles = 18 * 1024;   // matrices of the axes that a block stages in shared memory
 
 typedef unsigned long long SmallTag;
 struct __align__(16) SmallCell {
@@ -718,9 +721,18 @@ template <class Model, int M>
 cudaError_t small_launch(const StepArgs& a, const SmallArgs& s, int blocks, int threads, size_t smem, cudaStream_t st)
 {
     const void* k = (const void*)k_small_step<Model, M>;
-    if (smem > 40 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // The opt-in to more than 48 KB of shared memory (which the kernel's own arrays count towards), once per kernel
+    // and device and for the largest step, so that no other thread's smaller mesh takes it back before the launch.
+    static std::atomic<unsigned long long> opted{0};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const unsigned long long bit = 1ULL << (dev & 63);
+    if (smem > 0 && (dev > 63 || !(opted.load(std::memory_order_acquire) & bit))) {
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(sizeof(double) * (kSmallStageDoubles + 3 * 512)));
         if (e != cudaSuccess) return e;
+        opted.fetch_or(bit, std::memory_order_release);
     }
     void* args[] = {const_cast<StepArgs*>(&a), const_cast<SmallArgs*>(&s)};
     return cudaLaunchCooperativeKernel(k, dim3(blocks), dim3(threads), args, smem, st);
