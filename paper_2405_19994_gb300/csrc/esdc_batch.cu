@@ -54,7 +54,9 @@ namespace {
 std::mutex g_bconst_mu;
 bool g_bconst_done[64] = {false};
 
-constexpr int kMaxBlockTissues = 128;     // tissues one CG block may touch
+// Tissues one solve block may touch: 128 where its warps take whole tiles, and one more where they take pieces of
+// tiles (a block's range begins in the same tile as with whole ones and may end inside the next).
+constexpr int kTileBlockTissues = 128, kMaxBlockTissues = kTileBlockTissues + 1;
 
 // ---------------------------------------------------------------- kernels
 template <class Model>
@@ -1039,10 +1041,10 @@ int grid_nodes(const esdc_batch* b, int occ, int waves)
 // Pieces of a tile that the solve's warps take one by one.
 int solve_subs(const esdc_batch* b) { return b->opt.solver == 0 ? kSubs : 1; }
 
-// Largest number of tissues one solve block touches for a grid of nb blocks.
-int max_block_tissues(const esdc_batch* b, int nb, int threads)
+// Largest number of tissues one solve block touches for a grid of nb blocks whose warps take tiles in subs pieces.
+int max_block_tissues(const esdc_batch* b, int nb, int threads, int subs)
 {
-    const int nwb = threads / 32, subs = solve_subs(b);
+    const int nwb = threads / 32;
     const long long nwt = (long long)nb * nwb, n = (long long)subs * b->ntiles;
     int worst = 0;
     for (int blk = 0; blk < nb; ++blk) {
@@ -1070,7 +1072,7 @@ int cg_grid(const esdc_batch* b, int threads, int per_sm_wanted)
     long long nb = (long long)b->sms * per_sm;
     const long long need = ((long long)solve_subs(b) * b->ntiles + threads / 32 - 1) / (threads / 32);
     nb = std::max(1LL, std::min(nb, need));
-    while (nb > 1 && max_block_tissues(b, (int)nb, threads) > kMaxBlockTissues) --nb;
+    while (nb > 1 && max_block_tissues(b, (int)nb, threads, solve_subs(b)) > kMaxBlockTissues) --nb;
     return (int)nb;
 }
 
@@ -1155,7 +1157,7 @@ int bstep_grid(const esdc_batch* b, int M)
     long long nb = (long long)b->sms * std::min(occ, b->p_threads == 256 ? 2 : 1);
     const long long need = ((long long)solve_subs(b) * b->ntiles + b->p_threads / 32 - 1) / (b->p_threads / 32);
     nb = std::max(1LL, std::min(nb, need));
-    while (nb > 1 && max_block_tissues(b, (int)nb, b->p_threads) > kMaxBlockTissues) --nb;
+    while (nb > 1 && max_block_tissues(b, (int)nb, b->p_threads, solve_subs(b)) > kMaxBlockTissues) --nb;
     return (int)nb;
 }
 
@@ -1548,7 +1550,11 @@ int esdc_batch_create(int n, const esdc_mesh* meshes, const double* sigma, doubl
     cudaMemset(b->flags, 0, sizeof(int));
     auto_shape(b);
     if (b->cg_blocks < 1) return fail(ESDC_ERR_CUDA);
-    if (max_block_tissues(b, b->cg_blocks, b->cg_launch) > kMaxBlockTissues) return fail(ESDC_ERR_UNSUPPORTED);
+    // Every launch shape must do (esdc_batch_set_shape, _set_persistent, _tune), so the one with the fewest blocks
+    // decides, 512 threads and a block per SM, the automatic one with more blocks does not.
+    if (max_block_tissues(b, std::min(b->sms, (b->ntiles + 15) / 16), 512, 1) > kTileBlockTissues ||
+        max_block_tissues(b, b->cg_blocks, b->cg_launch, solve_subs(b)) > kMaxBlockTissues)
+        return fail(ESDC_ERR_UNSUPPORTED);
     if (cudaDeviceSynchronize() != cudaSuccess) return fail(ESDC_ERR_CUDA);
     *out = b;
     return ESDC_OK;
@@ -1779,7 +1785,7 @@ int esdc_batch_set_shape(esdc_batch* b, int node_waves, int cg_threads, int cg_b
         return set_berr(b, ESDC_ERR_INVALID_ARG, "launch shape out of range");
     const int nb = cg_grid(b, cg_threads, cg_blocks_per_sm);
     if (nb < 1) return set_berr(b, ESDC_ERR_CUDA, "CG occupancy query failed");
-    if (max_block_tissues(b, nb, cg_threads) > kMaxBlockTissues)
+    if (max_block_tissues(b, nb, cg_threads, solve_subs(b)) > kMaxBlockTissues)
         return set_berr(b, ESDC_ERR_UNSUPPORTED, "too many tissues per CG block for this shape");
     cudaDeviceSynchronize();
     drop_graph(b);

@@ -88,3 +88,34 @@ def test_largest_iteration_caps(cap):
         got, it_n = run(wls, persistent=persistent, cg_maxit=cap)[0]
         assert it.min() >= 1 and np.array_equal(it, it_n)
         assert all(np.array_equal(a, b) for a, b in zip(got, want))
+
+
+def test_most_tissues_of_every_launch_shape():
+    # 128 single-tile tissues per block of one 512-thread block per SM, but for the last: a block whose warps take
+    # quarters of tiles touches 129
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    w = I.hh_sheet_32().with_mesh(3, 2, 1)
+    w.boxes = np.array([[0, 1, 0, 1, 0, 1]], np.int32)
+    b = P.Batch.from_workloads([w] * (128 * sms - 1), M_max=1)
+    y0, y = b.new_state(), b.new_state()
+    b.init_state(y0, -70.0)
+    y0[0] += torch.rand(y0.shape[1], dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+    y.copy_(y0)
+    b.sweep(y, 0.0, w.dt, 1, 2)
+    assert b.residual()[0] == 0
+    want = y.clone()
+    for shape in ((1, 512, 1), (1, 256, 1)):
+        b.set_shape(*shape)
+        y.copy_(y0)
+        b.sweep(y, 0.0, w.dt, 1, 2)
+        assert b.residual()[0] == 0 and torch.equal(y, want)
+    for threads in (512, 256):
+        b.set_persistent(True, threads, 128)
+        y.copy_(y0)
+        b.sweep(y, 0.0, w.dt, 1, 2)
+        assert b.residual()[0] == 0 and torch.equal(y, want)
+    b.close()
+    # a batch that one of the shapes cannot take is refused
+    with pytest.raises(P.EsdcError) as e:
+        P.Batch.from_workloads([w] * (256 * sms), M_max=1)
+    assert e.value.code == -6
