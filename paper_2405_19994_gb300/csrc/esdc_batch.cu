@@ -487,10 +487,11 @@ __global__ void __launch_bounds__(512) k_cgb(BCgArgs a)
 // bytes take 40; an FP32 pass moves half the bytes and leaves that pipe alone.
 // 64 tissues of 64..512 nodes a side 32.3 -> 28.3 ms per step, 16 slices of 256x256 10.5 -> 9.0 ms per
 // Q^par solve.
-// A correction reduces the residual by 3e-6 at most (kFmin2; FP32's rounding
-// leaves about kappa 6e-8, kappa at most 64), so a warm-started solve takes one
-// or two.  The last one's FP32 residual tells whether it met the test, with
-// 2e-6 ||r|| as the allowance for its rounding; else the FP64 residual decides.
+// A correction is asked to reduce the residual by 3e-6 at most (kFmin2; FP32's
+// rounding leaves up to kappa 1e-7, kappa at most 64), so a warm-started solve
+// takes one or two.  The last one's FP32 residual tells whether it met the test,
+// with kappa 1e-7 ||r|| (at least 2e-6) as the allowance for its rounding
+// (ESDC_REF_ALLOW_KAPPA); else the FP64 residual decides.
 // What FP32 cannot do (a residual out of its range, no progress) the FP64
 // iterations finish (kStart64, kFp64).  The defect pass and its barrier are
 // what it costs, so small tissues, which the barriers bound, stay in FP64; the
@@ -817,7 +818,8 @@ __device__ bool cheb_all(const BCgArgs& a, unsigned& target)
             if (!isfinite(rr)) {
                 stop_tissue(k, ESDC_FLAG_NONFINITE);
             } else if (mode == kFp32) {
-                if (s_final[k] && sqrt(rr) + 2e-6 * sqrt(s_rr[k]) <= sqrt(s_stop[k])) stop_tissue(k, 0);
+                const double allow = fmax(ESDC_REF_ALLOW_MIN, ESDC_REF_ALLOW_KAPPA * (1.0 + 2.0 * s_delta[k]));
+                if (s_final[k] && sqrt(rr) + allow * sqrt(s_rr[k]) <= sqrt(s_stop[k])) stop_tissue(k, 0);
                 else s_mode[k] = kDefect;
             } else if (rr <= s_stop[k]) {
                 stop_tissue(k, 0);

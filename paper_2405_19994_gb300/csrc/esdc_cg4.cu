@@ -536,12 +536,12 @@ __global__ void __launch_bounds__(cheb_threads<LAY>(), 1) k_cheb4(CgArgs a, Cheb
 // nodes on it is the faster one (600x500 scalar sheet 2.21 / 2.19 ms per step,
 // 128x128x64 layered slab 7.32 / 5.35; 300x250 sheet 0.97 / 1.28, barrier-bound).
 //
-// A correction reduces the residual by 3e-6 at most (FP32 rounding leaves about
-// kappa 6e-8) and the passes share the reduction that the stop test needs, so a
+// A correction is asked to reduce the residual by 3e-6 at most (FP32 rounding leaves
+// up to kappa 1e-7) and the passes share the reduction that the stop test needs, so a
 // warm-started solve takes two.  The last correction's own FP32 residual tells
-// whether it met the test, with 2e-6 ||r|| (the residual it started from) as the
-// allowance for its rounding; else the FP64 residual decides and the passes go
-// on.  What refinement cannot do (residuals near FP32's range, no progress) the
+// whether it met the test, with kappa 1e-7 ||r|| (the residual it started from; at
+// least 2e-6) as the allowance for its rounding (ESDC_REF_ALLOW_KAPPA); else the
+// FP64 residual decides and the passes go on.  What refinement cannot do (residuals near FP32's range, no progress) the
 // FP64 iterations finish.  The result has FP64's error: every correction but the
 // last is measured by an FP64 residual, and the last one's rounding (1e-7 of a
 // correction of 1e-9 and below) is under x's own.
@@ -549,6 +549,7 @@ struct RefArgs {
     float *r, *z, *p, *q, *e;
     double qq[ESDC_CHEB_TAB];       // 4 q^{2 (k + 1)}
     double fmin2;                   // least reduction (squared) asked of one correction
+    double allow;                   // what its FP32 residual may miss, in units of the residual it started from
 };
 #define ESDC_REF_MAXOUT 8
 
@@ -657,7 +658,7 @@ __global__ void __launch_bounds__(cheb_threads<LAY>(), 1) k_cheb4_ref(CgArgs a, 
         double r32[1];
         grid_total<1>(part, 4 + (outer & 1), r32);
         if (!isfinite(r32[0])) { fp32 = false; break; }        // x and a.r are untouched: FP64 from here
-        if (final && sqrt(r32[0]) + 2e-6 * sqrt(rr) <= sqrt(stop)) {
+        if (final && sqrt(r32[0]) + f.allow * sqrt(rr) <= sqrt(stop)) {
             for (int qi = q0 + (int)threadIdx.x; qi < q1; qi += blockDim.x) {
                 const Q4<float> e = ld4(f.e + 4 * qi);
                 Q4<double> x = ld4(a.x + 4 * qi);
@@ -1126,6 +1127,8 @@ static cudaError_t cheb_launch(const CgArgsHost& h, const ChebArgs& c, bool ref,
     RefArgs f;
     f.r = h.w.r32; f.z = h.w.z32; f.p = h.w.p32; f.q = h.w.q32; f.e = h.w.e32;
     f.fmin2 = 1e-11;
+    const double sk = (1.0 + c.q) / (1.0 - c.q);                  // sqrt(kappa)
+    f.allow = std::fmax(ESDC_REF_ALLOW_MIN, ESDC_REF_ALLOW_KAPPA * sk * sk);
     double q2 = 1.0;
     for (int i = 0; i < ESDC_CHEB_TAB; ++i) {
         q2 *= c.q * c.q;
