@@ -78,14 +78,28 @@ CLASS_BYTES = {"setup": 3256.0, "node_sweep": 7464.0, "dct_solve": 120.0, "cheb_
                "residual": 2904.0}
 
 
+# Nodes between which a Chebyshev solve runs k_cheb4, whose iterations cheb_iter counts: at most 512 per SM run
+# k_small_solve, and from 400,000 on FP32 corrections (k_cheb4_ref) take the iterations' place.
+CHEB4_NODES = (152 * 512 + 1, 399999)
+
+
+def solve_class(solver_in_use: str, nodes: int) -> str:
+    """The solve class whose work per iteration has been counted ("dct", "cheb" or "cg"), or "uncounted"."""
+    if solver_in_use == "cheb" and not CHEB4_NODES[0] <= nodes <= CHEB4_NODES[1]:
+        return "uncounted"
+    return solver_in_use
+
+
 def class_work(solver_kind: str, K: int, it_mean: float, M: int = 4, fused: bool = True) -> dict:
-    """(FP64 instructions, bytes) per node and step of each kernel class; with
-    `fused`, the first sweep's node 1 belongs to the set-up launch."""
+    """(FP64 instructions, bytes) per node and step of each kernel class, None where they have not been
+    counted; with `fused`, the first sweep's node 1 belongs to the set-up launch."""
     solves = M * K
     if solver_kind == "dct":
         sv = (CLASS_FP64_OPS["dct_solve"] * solves, CLASS_BYTES["dct_solve"] * solves)
+    elif solver_kind in ("cheb", "cg"):
+        sv = (CLASS_FP64_OPS[solver_kind + "_iter"] * it_mean * solves, CLASS_BYTES[solver_kind + "_iter"] * it_mean * solves)
     else:
-        sv = (CLASS_FP64_OPS["cheb_iter"] * it_mean * solves, CLASS_BYTES["cheb_iter"] * it_mean * solves)
+        sv = (None, None)
     n1 = (NODE1["fp64_ops"], NODE1["bytes"]) if fused else (0.0, 0.0)
     return {"setup": (CLASS_FP64_OPS["setup"] + n1[0], CLASS_BYTES["setup"] + n1[1]),
             "node": (CLASS_FP64_OPS["node_sweep"] * K - n1[0], CLASS_BYTES["node_sweep"] * K - n1[1]),
@@ -356,7 +370,7 @@ def run_ours(args):
     roof = {"kernel": dom}
     node_launches_step = prof["node"][1] / args.steps if prof["node"][1] else 0
     fused = abs(node_launches_step - K * M) < 0.5                # node 1 inside the launch before it
-    if dom == "node" and M in NODE_FLOPS_PER_SWEEP and args.precision == "fp64":
+    if dom == "node" and M in NODE_FLOPS_PER_SWEEP and args.precision == "fp64" and prof["setup"][1]:
         # per launch: the node class's work per step over its launches per step
         flops = (NODE_FLOPS_PER_SWEEP[M] * K - (NODE1["flops"] if fused else 0.0)) * N / node_launches_step
         byts = (NODE_BYTES_PER_SWEEP[M] * K - (NODE1["bytes"] if fused else 0)) * N / node_launches_step
@@ -378,9 +392,9 @@ def run_ours(args):
                      "hbm_peak_gbs": peaks["hbm_gbs"]})
     else:
         bytes_launch = None
-        if dom == "cg":
+        if dom == "cg" and solve_class(solver.solver_in_use(), N) == "cg":
             bytes_launch = (CG_BYTES_PER_NODE_ITER * it_mean + CG_BYTES_PER_NODE_SETUP) * N
-        elif dom == "node":
+        elif dom == "node" and prof["setup"][1]:
             bytes_launch = NODE_BYTES_PER_SWEEP.get(M, 7464) * K * N / max(node_launches_step, 1)
         ach = bytes_launch / (per_launch_ms[dom] * 1e-3) / 1e9 if bytes_launch else None
         roof.update({"bound": "hbm", "unit": "GB/s", "achieved": ach, "peak": peaks["hbm_gbs"],
@@ -388,15 +402,17 @@ def run_ours(args):
                      "traffic": None})
     if args.precision == "fp64" and M == 4:
         classes = {}
-        for cls, (ops, byts) in class_work(solver_kind, K, it_mean, fused=fused).items():
+        one_launch = prof["setup"][1] == 0 and prof["cg"][1] == 0          # the whole step under "node"
+        for cls, (ops, byts) in class_work(solve_class(solver.solver_in_use(), N), K, it_mean, fused=fused).items():
             sec = prof[cls][0] * 1e-3 / args.steps
             if sec <= 0:
                 continue
-            rate = ops * N / sec
-            classes[cls] = {"ms_per_step": sec * 1e3, "fp64_ops_per_node_step": ops,
-                            "fp64_issue_frac": rate / FP64_ISSUE_PEAK,
-                            "bytes_per_node_step": byts, "gbs": byts * N / sec / 1e9,
-                            "hbm_frac": byts * N / sec / 1e9 / peaks["hbm_gbs"]}
+            counted = ops is not None and not one_launch
+            gbs = byts * N / sec / 1e9 if counted else None
+            classes[cls] = {"ms_per_step": sec * 1e3, "fp64_ops_per_node_step": ops if counted else None,
+                            "fp64_issue_frac": ops * N / sec / FP64_ISSUE_PEAK if counted else None,
+                            "bytes_per_node_step": byts if counted else None, "gbs": gbs,
+                            "hbm_frac": gbs / peaks["hbm_gbs"] if counted else None}
         roof["classes"] = classes
         roof["classes_note"] = (
             "fp64_issue_frac: FP64 instructions (DFMA, DADD, DMUL; counted by ncu per node, profiles/) per second "
