@@ -484,9 +484,8 @@ __global__ void __launch_bounds__(512) k_cgb(BCgArgs a)
 // take each off the FP64 residual (kDefect: r -= B e) and add it to x in FP64,
 // to the same stop test.  An FP64 pass costs 10 FP64-pipe operations per node,
 // 85 us for the 64 tissues of 64 to 512 nodes a side (5.1M nodes) where its
-// bytes take 40; an FP32 pass moves half the bytes and leaves that pipe alone.
-// 64 tissues of 64..512 nodes a side 32.3 -> 28.3 ms per step, 16 slices of 256x256 10.5 -> 9.0 ms per
-// Q^par solve.
+// bytes take 40; an FP32 pass moves half the bytes and leaves that pipe alone
+// (the figures per step are at kRefMinNodes).
 // A correction is asked to reduce the residual by 3e-6 at most (kFmin2; FP32's
 // rounding leaves up to kappa 1e-7, kappa at most 64), so a warm-started solve
 // takes one or two.  The last one's FP32 residual tells whether it met the test,
@@ -497,12 +496,18 @@ __global__ void __launch_bounds__(512) k_cgb(BCgArgs a)
 // what it costs, so small tissues, which the barriers bound, stay in FP64; the
 // line depends on the tissue alone, as its results do.
 enum : int { kStop = 0, kFp64, kFp32, kDefect, kStart64 };
-constexpr int kRefMinNodes = 16385;      // nodes of a tissue from which it iterates in FP32
+// Nodes of a tissue from which it iterates in FP32.  What pays is work per SM, so the better line depends on how many
+// tissues there are, but a tissue's results may not: FP32 / FP64 passes, ms per step (HH, M = 3, K = 4) of 64, 16, 8
+// and 1 tissues of 128x128: 5.87 / 6.32, 2.25 / 2.17, 1.69 / 1.44, 1.19 / 1.02; of 160x128: 6.71 / 7.88, 2.80 / 2.81,
+// 1.88 / 1.64, 1.22 / 1.04; of 256x256: 18.7 / 22.9, 5.85 / 6.35, 3.42 / 3.55, 1.39 / 1.18.
+constexpr int kRefMinNodes = 16385;
 constexpr int kRefMaxOut = 8;            // corrections before the FP64 iterations take over
 constexpr double kFmin2 = 1e-11;         // least reduction (squared) asked of one correction
 // A warp takes pieces of 128 nodes, a quarter of a tile, each with its own partial sums: one warp
 // gets an FP64 instruction through every 64 cycles, so 16 nodes per lane took 5 us per pass where a
-// batch has fewer tiles than the GPU has warps (four of an SM's warps keep its pipe busy).
+// batch has fewer tiles than the GPU has warps (four of an SM's warps keep its pipe busy): 8 slices
+// of 128x128 in two-level HSDC 11.7 -> 7.9 ms, 64 tissues of 64..512 a side 27.2 -> 26.6; 16 slices of 256x256 under
+// Q^par, which had a warp per tile already, pay for the look-ups: 8.72 -> 9.06.
 constexpr int kSubs = 4, kSubNodes = ESDC_TILE / kSubs;
 
 __device__ bool cheb_all(const BCgArgs& a, unsigned& target)
@@ -841,8 +846,10 @@ __device__ bool cheb_all(const BCgArgs& a, unsigned& target)
 
 // PER_SM: blocks of 512 threads that the registers allow per SM.  One (104 registers, more loads
 // in flight per warp) while a 512-thread block per SM has a warp for every tile, else two (64; or
-// four of 256): 16 slices of 256x256 (2048 tiles) 9.12 / 9.28 ms per Q^par solve, 64 tissues of
-// 64..512 nodes a side (9,900 tiles) 31.4 / 28.5 ms per step.
+// four of 256).  ms per step with one / four of 256 (HH, M = 3, K = 4) of n tissues of 256x256: 64
+// (8192 tiles) 20.97 / 18.71, 32 10.38 / 9.69, 20 7.06 / 6.72; below the line of 16 tiles per SM, which was set
+// when a warp took whole tiles, four are the faster ones too by now: 19 6.48 / 6.14, 16 5.85 / 5.44, 8
+// 3.43 / 3.36.  Of 128x128: 160 14.54 / 14.89, 96 9.27 / 9.24, 48 4.97 / 5.13.
 template <int PER_SM>
 __global__ void __launch_bounds__(512, PER_SM) k_chebb(BCgArgs a)
 {
@@ -984,7 +991,7 @@ struct esdc_batch {
     unsigned long long* rmax = nullptr;    // [ntis][2 NS]
     // launch shapes (esdc_batch_tune)
     int node_waves = 1, cg_threads = 512, cg_blocks = 0;
-    int cg_launch = 512;                   // threads per solve block: cg_threads, or auto_threads
+    int cg_launch = 512;                   // threads per solve block: cg_threads, or what auto_shape gives
     int occ_node[ESDC_MMAX + 1] = {0}, occ_setup[ESDC_MMAX + 1] = {0}, occ_res[ESDC_MMAX + 1] = {0},
         occ_iter[ESDC_MMAX + 1] = {0};
     // one persistent launch per step (k_bstep; Chebyshev solves only): on/off,
@@ -1080,8 +1087,8 @@ int cg_grid(const esdc_batch* b, int threads, int per_sm_wanted)
 
 // The solve's shape until esdc_batch_set_shape gives one.  A warp takes whole pieces of tiles: one
 // block per SM with as many warps as give every SM its share, or, above 16 tiles per SM, four
-// 256-thread blocks per SM (their barriers' waits overlap: 64 tissues of 64..512 nodes a side 27.0
-// ms per step against 28.4 with two blocks of 512).  With 512-thread blocks throughout, the 32
+// 256-thread blocks per SM (their barriers' waits overlap: 64 tissues of 64..512 nodes a side 26.6
+// ms per step against 28.1 with two blocks of 512, 30.4 with two of 256 and 31.4 with one of 512).  With 512-thread blocks throughout, the 32
 // tiles of a 128x128 sheet ran on two of the 152 SMs.
 void auto_shape(esdc_batch* b)
 {

@@ -531,8 +531,10 @@ __global__ void __launch_bounds__(cheb_threads<LAY>(), 1) k_cheb4(CgArgs a, Cheb
 // off the FP64 residual (r -= B e in FP64, e widened exactly) and added to x in
 // FP64.  An FP64 iteration of a large mesh costs its 13 (scalar) to 19 (layered)
 // FP64-pipe operations per node: 110 us at 4.2M nodes where its bytes take 30.
-// The FP32 iteration moves 24 bytes per node and leaves the FP64 pipe alone:
-// 1293 -> 530 us per solve of the 256x256x64 layered slab, and from 305,000 to 350,000
+// The FP32 iteration moves 24 bytes per node and leaves the FP64 pipe alone; what
+// bounds the solve then is the FP64 passes' issue (pipe 58% busy over a solve at 4.2M
+// nodes, 46% at 1M) and 16 warps per SM waiting on loads, shared memory and barriers,
+// with L2 at 23% and DRAM at 14% of their peaks.  1293 -> 540 us per solve of the 256x256x64 layered slab, and from 305,000 to 350,000
 // nodes on it is the faster one (600x500 scalar sheet 2.21 / 2.19 ms per step,
 // 128x128x64 layered slab 7.32 / 5.35; 300x250 sheet 0.97 / 1.28, barrier-bound).
 //

@@ -381,7 +381,7 @@ __device__ __forceinline__ void setup_body(const StepArgs& a, const PhaseArgs& p
                                    // the FP64 pipe, the kernel waits on memory and on integer work: 5 / 6 /
                                    // 7 / 8 blocks take 11.14 / 10.36 / 10.15 / 10.25 ms per step on the 128x128x32
                                    // SYN19 slab, 4.85 / 4.77 / 4.15 / 4.24 on 90x75x19, 9.09 / 9.00 / 8.72 / 8.75 per
-                                   // Q^par solve of 16 256x256 slices
+                                   // Q^par solve of 16 256x256 slices (9.1 since the solves' 128-node pieces)
 #endif
 // TAU: batched kernels may add the FAS correction tau (a.tau, rows 1..M; the
 // recursive form adds tau_i - tau_{i-1}, tau_0 = 0, to every row of node i).

@@ -10,15 +10,21 @@ std::mutex g_const_mu;
 bool g_const_done[64] = {false};
 
 // Nodes per block up to which a step runs as one launch (N <= SMs times that).
-// Against the launch sequence (us per step, HH M = 3 K = 4): 4,096 nodes 288 / 745,
-// 16,384 601 / 793, 30,000 514 / 843; 75,000 nodes (512 per block, one role, 16
-// warps' FP64 issue) 1042 / 952, 65,536 SYN19 nodes 3.09 / 2.82 ms, 72,000 layered
-// 1446 / 1051.  A conductivity field's sequence has the slower solve: 65,536 nodes
-// 1084 / 1288.
+// One launch against the sequence with k_small_solve (us per step, HH M = 3 K = 4 /
+// SYN19 M = 4 K = 6): scalar sheets of 7,575 nodes 332 / 435 and 859 / 1324, 21,000 462 /
+// 492 and 1263 / 1500, 38,805 494 / 548 and 1564 / 1918; above the line (512 nodes per
+// block, one role, 16 warps' FP64 issue) 42,000 nodes 846 / 634, 77,000 939 / 706, SYN19
+// 65,536 2923 / 2412.  The line is late for what has more neighbours: 37,800 layered nodes
+// 616 / 609 (SYN19 1941 / 2079), 38,805 of the fourth order 745 / 652.
+// Fields have a line of their own from when the sequence solved them with k_cheb (65,536
+// nodes 1084 / 1288); with k_small_solve the sequence is the faster one above 256 nodes
+// per SM for them too: 42,000 nodes 940 / 711, 65,536 974 / 767 and SYN19 3287 / 2690.
 constexpr int kSmallNodes = 256, kSmallNodesField = 512;
 // Dense cosine products against the sequence's FFT passes: N sum(n + 2) FP64
-// operations per solve over two lanes per SM and clock.  128x128 (14,000 cycles) 601
-// against 793 us per step; 256x256 would be 111,000 cycles, four times the FFT solve.
+// operations per solve over two lanes per SM and clock (us per step, HH / SYN19 as
+// above).  128x128 (14,000 cycles) 587 against 696 and 1239 / 1779, 64x32x16 (12,500) 445 / 700,
+// 256x64 (17,500) 710 / 672 and 1664 / 1728; above the line 256x128 (42,000) 802 / 746 and
+// 2360 / 2170; 256x256 would be 111,000 cycles, four times the FFT solve.
 constexpr double kSmallDctCycles = 40000.0;
 constexpr int kSmallDctAxis = 256;
 constexpr int kSmallDctCable = 128;         // 1D: one line means one block
