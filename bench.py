@@ -903,7 +903,8 @@ def run_batch_form(args):
         cel = time.perf_counter() - c0
         cpu = {"value": done / cel, "unit": UNIT, "cores": oracle.oracle.threads(), "kind": "oracle",
                "sample": "2 steps from rest of each of the first 4 tissues of the batch"}
-    launches_per_step = 1 + K * (M + 1) + K * M + 1
+    # set-up, K M node launches (node 1 runs inside the launch before it), K M solves, residual; or one launch
+    launches_per_step = 1 if pers[0] else 1 + K * M + K * M + 1
     # ---- Batch B: P = 16 time slices x M = 3 of one 512 x 512 tissue under Q^par
     qb = run_qpar_batch(args, P, I, torch, timed)
     line = {

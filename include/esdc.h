@@ -462,7 +462,7 @@ int esdc_adjoint_backward(esdc_handle* h, const double* ckpt, double t0, double 
  * cover all tissues, and each diffusion solve is one cooperative launch that
  * runs all tissues' CG iterations side by side, each with its own step sizes
  * and stop test.  The launches of a step are recorded once in a CUDA graph and
- * replayed.  Every reduction is fixed per 512-node tile and per tissue, so a
+ * replayed.  Every reduction is fixed per tile of 512 nodes and per tissue, so a
  * tissue's results are identical bit for bit whatever the rest of the batch and
  * whatever launch shape the autotuner picks.  The paper batches its
  * time-parallel slices across processors (Sec. 3.2); batching tissues is this

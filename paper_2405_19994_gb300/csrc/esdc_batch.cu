@@ -7,9 +7,10 @@
 // tile of 512 nodes belongs to exactly one tissue.  Node kernels find a node's
 // tissue from its tile and skip the padding at the end of each tissue.
 //
-// Determinism.  Every dot product of the solves is reduced first over one tile, in
-// an order fixed by the tile alone (lane l of a warp adds nodes l, l+32, ...,
-// then a fixed shuffle tree), then over the tiles of the tissue in tile order.
+// Determinism.  Every dot product of the solves is reduced first over one tile (the
+// Chebyshev solves: over a quarter of one), in an order fixed by the tile alone (lane l
+// of a warp adds nodes l, l+32, ..., then a fixed shuffle tree), then over those
+// sums of the tissue in order.
 // The result of every tissue is therefore independent of which other tissues
 // share the batch and of the launch shape (blocks, threads, tiles per warp);
 // the residual norms are maxima and order-free.  A batch of many tissues gives
@@ -864,7 +865,7 @@ __global__ void __launch_bounds__(512, PER_SM) k_chebb(BCgArgs a)
 // (cheb_all), then the residual.  Phases are separated by the bounded grid
 // barrier.  Each phase does exactly the arithmetic of the corresponding kernel
 // of the launch sequence (the node bodies are per node; the solve's
-// reductions are fixed by the 512-node tiles), so the results are bit for bit
+// reductions are fixed by the quarters of the 512-node tiles), so the results are bit for bit
 // those of the sequence whatever the grid, block size or node tile.
 struct BStepArgs {
     int K;
